@@ -313,6 +313,7 @@ void launch_scale(size_t count, const double *factor, T *x, cudaStream_t s);
 struct GramPlan {
     long n;
     int na, nb, tiles_a, tiles_b, ntiles, chunks;
+    int edge;          // columns per tile (<= 64)
     long chunk_rows;
     bool sym;
 };

@@ -10,9 +10,9 @@
 namespace hq {
 
 // ---------------------------------------------------------------------------
-// Gram: out = w [A1 A2]^T [B1 B2], tiles of 64 x 64, split over point chunks.
+// Gram: out = w [A1 A2]^T [B1 B2], tiles of at most 64 x 64, split over point chunks.
 // ---------------------------------------------------------------------------
-constexpr int GT = 64;   // tile edge
+constexpr int GT = 64;   // largest tile edge
 constexpr int GK = 16;   // points per smem stage
 
 GramPlan make_gram_plan(long n, int na, int nb, bool sym) {
@@ -23,6 +23,8 @@ GramPlan make_gram_plan(long n, int na, int nb, bool sym) {
     p.sym = sym;
     p.tiles_a = (na + GT - 1) / GT;
     p.tiles_b = (nb + GT - 1) / GT;
+    // columns per tile: the blocks' columns split evenly over their tiles
+    p.edge = std::max((na + p.tiles_a - 1) / p.tiles_a, (nb + p.tiles_b - 1) / p.tiles_b);
     p.ntiles = sym ? p.tiles_a * (p.tiles_a + 1) / 2 : p.tiles_a * p.tiles_b;
     long target = std::max(1L, (long)(2 * 152) / p.ntiles);
     long maxchunks = std::max(1L, (n + GT - 1) / GT);
@@ -59,78 +61,121 @@ __device__ __forceinline__ T gat(const T *X1, int n1, const T *X2, int n2, long 
     return c < n1 ? X1[(size_t)p * n1 + c] : X2[(size_t)p * n2 + (c - n1)];
 }
 
-template <typename T>
+// One tile over one point chunk: 16 x 16 threads of R x R entries (rows ty + 16 i,
+// columns tx + 16 j), tile edge 16 R.  R is the smallest of 1 .. 4 that covers
+// the tiles (tile_edge): the FP64 pipe bounds the kernel, so entries beyond
+// the blocks' columns cost as much as the others (a 64 x 64 tile for 32
+// columns did four times the work).  The diagonal tiles of a symmetric Gram
+// form their sub-blocks on and above the diagonal only (10 of 16 at R = 4).
+// The next stage's loads are issued before the products of this one.  Every
+// entry is summed over the points in order, whatever R.
+// Measured, 48^3 points (before: always 64 x 64 tiles): 16 x 16 columns 807 -> 99,
+// 32 x 32 806 -> 239, 64 x 64 842 -> 792 us, symmetric 798 -> 517 us; the FP64 pipe
+// alone takes 165 us for 32 x 32.
+template <typename T, int R, bool DIAG>
+__device__ __forceinline__ void gram_tile_products(const T (&As)[GK][GT + 1], const T (&Bs)[GK][GT + 1],
+                                                   int tx, int ty, T (&acc)[R][R]) {
+#pragma unroll
+    for (int kk = 0; kk < GK; kk++) {
+        T a[R], b[R];
+#pragma unroll
+        for (int i = 0; i < R; i++) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+        for (int j = 0; j < R; j++) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < R; i++)
+#pragma unroll
+            for (int j = DIAG ? i : 0; j < R; j++) acc[i][j] += a[i] * b[j];
+    }
+}
+
+template <typename T, int R>
 __global__ void __launch_bounds__(256) k_gram_partial(GramPlan P, const T *A1, int na1,
                                                       const T *A2, int na2, const T *B1,
                                                       int nb1, const T *B2, int nb2,
                                                       double *partials) {
+    constexpr int E = 16 * R;               // tile edge
+    constexpr int LD = GK * E / 256;        // values of each operand per thread and stage
     __shared__ T As[GK][GT + 1];
     __shared__ T Bs[GK][GT + 1];
     const int tile = blockIdx.x, chunk = blockIdx.y;
     int ta, tb;
     tile_of(tile, P.tiles_a, P.sym, ta, tb);
-    const int a0 = ta * GT, b0 = tb * GT;
+    const bool diag = P.sym && ta == tb;
+    const int a0 = ta * P.edge, b0 = tb * P.edge;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const long r0 = (long)chunk * P.chunk_rows;
     const long r1 = (P.n < r0 + P.chunk_rows) ? P.n : r0 + P.chunk_rows;
-    T acc[4][4];
+    T acc[R][R];
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < R; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = T(0);
+        for (int j = 0; j < R; j++) acc[i][j] = T(0);
+    T va[LD], vb[LD];
+    auto load = [&](long p0) {
+#pragma unroll
+        for (int u = 0; u < LD; u++) {
+            const int idx = threadIdx.x + 256 * u, kk = idx / E, c = idx % E;
+            const long p = p0 + kk;
+            const int ca = a0 + c, cb = b0 + c;
+            va[u] = (p < r1 && ca < P.na) ? gat(A1, na1, A2, na2, p, ca) : T(0);
+            vb[u] = (p < r1 && cb < P.nb) ? gat(B1, nb1, B2, nb2, p, cb) : T(0);
+        }
+    };
+    if (r0 < r1) load(r0);
     for (long p0 = r0; p0 < r1; p0 += GK) {
-        for (int idx = threadIdx.x; idx < GK * GT; idx += 256) {
-            int kk = idx / GT, c = idx % GT;
-            long p = p0 + kk;
-            int ca = a0 + c, cb = b0 + c;
-            As[kk][c] = (p < r1 && ca < P.na) ? gat(A1, na1, A2, na2, p, ca) : T(0);
-            Bs[kk][c] = (p < r1 && cb < P.nb) ? gat(B1, nb1, B2, nb2, p, cb) : T(0);
+#pragma unroll
+        for (int u = 0; u < LD; u++) {
+            const int idx = threadIdx.x + 256 * u;
+            As[idx / E][idx % E] = va[u];
+            Bs[idx / E][idx % E] = vb[u];
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GK; kk++) {
-            T a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] += a[i] * b[j];
-        }
+        if (p0 + GK < r1) load(p0 + GK);
+        if (diag) gram_tile_products<T, R, true>(As, Bs, tx, ty, acc);
+        else gram_tile_products<T, R, false>(As, Bs, tx, ty, acc);
         __syncthreads();
     }
-    double *dst = partials + ((size_t)chunk * P.ntiles + tile) * GT * GT;
+    double *dst = partials + ((size_t)chunk * P.ntiles + tile) * E * E;
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < R; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) dst[(ty + 16 * i) * GT + tx + 16 * j] = (double)acc[i][j];
+        for (int j = 0; j < R; j++)
+            if (!diag || i <= j) dst[(ty + 16 * i) * E + tx + 16 * j] = (double)acc[i][j];
 }
 
 // one thread per tile entry (grid: tiles x entry blocks), chunks summed in order
 __global__ void k_gram_reduce(GramPlan P, const double *partials, double w, double *out) {
-    const int tile = blockIdx.x;
+    const int tile = blockIdx.x, E = (P.edge + 15) / 16 * 16;
     int ta, tb;
     tile_of(tile, P.tiles_a, P.sym, ta, tb);
     const int e = blockIdx.y * blockDim.x + threadIdx.x;
-    if (e >= GT * GT) return;
-    const int la = e / GT, lb = e % GT;
-    const int a = ta * GT + la, b = tb * GT + lb;
-    if (a >= P.na || b >= P.nb) return;
-    double s = ordered_sum(partials + (size_t)tile * GT * GT + e, P.chunks, (size_t)P.ntiles * GT * GT);
+    if (e >= E * E) return;
+    const int la = e / E, lb = e % E;
+    const bool diag = P.sym && ta == tb;
+    if (diag && la > lb) return;   // its mirror entry's thread writes it
+    const int a = ta * P.edge + la, b = tb * P.edge + lb;
+    if (la >= P.edge || lb >= P.edge || a >= P.na || b >= P.nb) return;
+    double s = ordered_sum(partials + (size_t)tile * E * E + e, P.chunks, (size_t)P.ntiles * E * E);
     s *= w;
     out[(size_t)a * P.nb + b] = s;
-    if (P.sym && ta != tb) out[(size_t)b * P.nb + a] = s;
+    if (P.sym && a != b) out[(size_t)b * P.nb + a] = s;
 }
 
 template <typename T>
 void launch_gram(const GramPlan &p, const T *A1, int na1, const T *A2, int na2, const T *B1,
                  int nb1, const T *B2, int nb2, double w, double *partials, double *out,
                  cudaStream_t s) {
-    HQ_LAUNCH(HQ_K_GRAM, k_gram_partial<T><<<dim3(p.ntiles, p.chunks), 256, 0, s>>>(p, A1, na1, A2, na2, B1, nb1,
-                                                               B2, nb2, partials));
-    HQ_LAUNCH(HQ_K_GRAM, k_gram_reduce<<<dim3(p.ntiles, (GT * GT + 255) / 256), 256, 0, s>>>(
+    const dim3 grid(p.ntiles, p.chunks);
+    const int R = (p.edge + 15) / 16;
+    auto go = [&](auto kernel) {
+        HQ_LAUNCH(HQ_K_GRAM, kernel<<<grid, 256, 0, s>>>(p, A1, na1, A2, na2, B1, nb1, B2, nb2, partials));
+    };
+    if (R == 1) go(k_gram_partial<T, 1>);
+    else if (R == 2) go(k_gram_partial<T, 2>);
+    else if (R == 3) go(k_gram_partial<T, 3>);
+    else go(k_gram_partial<T, 4>);
+    HQ_LAUNCH(HQ_K_GRAM, k_gram_reduce<<<dim3(p.ntiles, (256 * R * R + 255) / 256), 256, 0, s>>>(
                              p, partials, w, out));
 }
 
