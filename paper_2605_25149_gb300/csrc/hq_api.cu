@@ -608,6 +608,29 @@ template <typename T>
 hq_status vcycle(hq_ctx *x, int l, const T *r, T *Zf, T *Tb, bool first_done, double *part_final,
                  const double *r64dot = nullptr);
 
+// w.r = restriction of r - A cur from level v to level w; res: scratch block of
+// level v.  Rows that fit one CTA: the residual and the x-restriction in one
+// pass, y and z in another; else the residual, then the 1-D passes.
+template <typename T>
+void resid_restrict(hq_ctx *x, Level &v, Level &w, const T *cur, const T *r, T *res) {
+    const T c = (T)v.c;
+    T *half = (T *)x->mxt1;
+    if (rows_fit<T>(v.m, w.m, x->N)) {
+        launch_resid_restrict_x<T>(v.m, w.m, x->N, v.tab, (const T *)v.Dt, c, cur, r, half, x->st);
+        launch_restrict_yz<T>(v.m, w.m, x->N, v.tab, half, (T *)w.r, x->st);
+        return;
+    }
+    launch_resid<T>(v.g, (const T *)v.Dt, c, cur, r, res, nullptr, nullptr, x->st);
+    launch_restrict<T>(v.m, w.m, x->N, v.tab, res, half, (T *)w.r, x->st);
+}
+
+// the first two sweeps of an FP32 V-cycle on level l run as one pass (the
+// first one from zero is wD r, formed on the fly)
+bool two_first_sweeps(const hq_ctx *x, int l) {
+    return (x->mixed || x->mg32) && l + 1 < x->L && x->cfg.mg_nu1 >= 2 &&
+           rows_fit<float>(x->mg[l].m, x->mg[l + 1].m, x->N);
+}
+
 // The FP64 V-cycle of level l with the smoothing sweeps from the pre-scaled
 // right-hand side rt = wD r (launch_jacobi_rt): the first sweep from zero is
 // rt itself (written by launch_jacobi_first, or by the PCG update when
@@ -645,10 +668,8 @@ hq_status vcycle_rt(hq_ctx *x, int l, const double *r, double *Zf, double *Tb, b
         cur = o;
     }
     double *res = next(cur);
-    launch_resid<double>(v.g, v.D, c, cur, r, res, nullptr, nullptr, x->st);
     Level &w = x->mg[l + 1];
-    launch_restrict<double>(v.m, w.m, x->N, v.tab, res, (double *)x->mxt1, (double *)x->mxt2,
-                            (double *)w.r, x->st);
+    resid_restrict<double>(x, v, w, cur, r, res);
     HQ_TRY(vcycle<double>(x, l + 1, (const double *)w.r, (double *)w.z, (double *)w.t, false,
                           nullptr));
     launch_prolong<double>(v.m, w.m, x->N, v.tab, (const double *)w.z, (double *)x->mxt1,
@@ -732,14 +753,22 @@ hq_status vcycle(hq_ctx *x, int l, const T *r, T *Zf, T *Tb, bool first_done, do
     }
     T *cur = first_target<T>(x, l, Zf, Tb);
     T *oth = (cur == Zf) ? Tb : Zf;
-    if (!first_done) launch_jacobi_first<T>(v.g, (const T *)v.wDt, r, cur, x->st);
-    for (int s = 1; s < x->cfg.mg_nu1; s++) {
+    int swept = 1;
+    if constexpr (std::is_same<T, float>::value) {
+        if (two_first_sweeps(x, l)) {
+            // the buffer two sweeps would end in: the order of the writes is unchanged
+            std::swap(cur, oth);
+            launch_sweep2(v.m, x->N, (const float *)v.wDt, c, omw, r, cur, x->st);
+            swept = 2;
+        }
+    }
+    if (swept == 1 && !first_done) launch_jacobi_first<T>(v.g, (const T *)v.wDt, r, cur, x->st);
+    for (int s = swept; s < x->cfg.mg_nu1; s++) {
         launch_jacobi<T>(v.g, (const T *)v.Dt, (const T *)v.wDt, c, omw, r, cur, oth, nullptr, x->st);
         std::swap(cur, oth);
     }
-    launch_resid<T>(v.g, (const T *)v.Dt, c, cur, r, oth, nullptr, nullptr, x->st);
     Level &w = x->mg[l + 1];
-    launch_restrict<T>(v.m, w.m, x->N, v.tab, oth, (T *)x->mxt1, (T *)x->mxt2, (T *)w.r, x->st);
+    resid_restrict<T>(x, v, w, cur, r, oth);
     HQ_TRY(vcycle<T>(x, l + 1, (const T *)w.r, (T *)w.z, (T *)w.t, false, nullptr));
     launch_prolong<T>(v.m, w.m, x->N, v.tab, (const T *)w.z, (T *)x->mxt1, (T *)x->mxt2, cur, oth,
                       x->st);
@@ -791,7 +820,7 @@ hq_status precondition(hq_ctx *x, const T *r, T *z, T *tbuf, bool first_done, do
 
 // the first damped-Jacobi sweep can be fused into the x / r update when the
 // V-cycle runs on the PCG's own buffers (more than one level, same precision)
-bool fuse_first_sweep(hq_ctx *x) { return x->L > 1 && !x->mg32; }
+bool fuse_first_sweep(hq_ctx *x) { return x->L > 1 && !x->mg32 && !two_first_sweeps(x, 0); }
 
 // FP64 block PCG with an FP32 V-cycle whose finest level runs as separate
 // kernels in linear point order: the FP64 <-> FP32 interface is fused into the
@@ -811,8 +840,8 @@ int prec_rows(hq_ctx *x) {
 }
 
 // the block PCG's preconditioner in mgf contexts: z (FP32, in Z32) = M r with
-// r32 written here (first_done false) or by k_pcg_xr_mg together with the
-// first sweep (first_done true); part: the FP64 partials of r.z
+// r32 written here (first_done false) or by k_pcg_xr_mg, with the first sweep
+// where it runs alone (first_done true); part: the FP64 partials of r.z
 hq_status precondition_mgf(hq_ctx *x, const double *r, bool first_done, double *part) {
     if (!first_done) launch_convert_d2f((size_t)x->n * x->N, r, x->R32, x->st);
     return vcycle<float>(x, 0, x->R32, x->Z32, x->T32, first_done, part, r);
@@ -886,7 +915,9 @@ hq_status pcg_half(hq_ctx *x, T *X, double rtol) {
     if constexpr (std::is_same<T, double>::value) {
         if (mgf(x)) {
             launch_pcg_xr_mg(g, sc.alpha, P, Q, X, R, x->part, (const float *)x->mg[0].wDt,
-                             x->R32, first_target<float>(x, 0, x->Z32, x->T32), x->st);
+                             x->R32,
+                             two_first_sweeps(x, 0) ? nullptr : first_target<float>(x, 0, x->Z32, x->T32),
+                             x->st);
             done = true;
         }
     }
@@ -2483,7 +2514,7 @@ hq_status smooth_impl(hq_ctx *x, int l, const void *r, const void *zin, void *zo
 template <typename T>
 hq_status restrict_impl(hq_ctx *x, int l, const void *rf, void *rc) {
     launch_restrict<T>(x->lev[l].m, x->lev[l + 1].m, x->N, x->lev[l].tab, (const T *)rf,
-                       (T *)x->xt1, (T *)x->xt2, (T *)rc, x->st);
+                       (T *)x->xt1, (T *)rc, x->st);
     return check_launch(x);
 }
 template <typename T>
@@ -2632,6 +2663,7 @@ hq_status hq_init(const hq_config *cfg, void *d_workspace, size_t bytes, void *c
     if (x->mixed) hq::tc_prepare();
     hq::lu_prepare();
     hq::vcoarse_prepare();
+    hq::rows_prepare();
     hq::lu32_prepare();
     if (x->ozimg || x->ozgram) hq::oz_prepare();
     if (e != cudaSuccess) {

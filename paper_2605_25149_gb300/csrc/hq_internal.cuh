@@ -130,15 +130,37 @@ struct XferTab {
     float *pwf;
 };
 void launch_xfer_tables(int mf, int mc, const XferTab &t, cudaStream_t s);
-// rc = ((mc+1)/(mf+1))^3 P^T rf, three 1-D passes through tmp1 (mf*mf*mc*N)
-// and tmp2 (mf*mc*mc*N)
+// rc = ((mc+1)/(mf+1))^3 P^T rf, the x pass through tmp1 (mf*mf*mc*N), then
+// y and z in one
 template <typename T>
-void launch_restrict(int mf, int mc, int N, const XferTab &t, const T *rf, T *tmp1, T *tmp2,
-                     T *rc, cudaStream_t s);
-// ef_out = ef_in + P ec, three 1-D passes through tmp2 and tmp1
+void launch_restrict(int mf, int mc, int N, const XferTab &t, const T *rf, T *tmp1, T *rc,
+                     cudaStream_t s);
+// ef_out = ef_in + P ec, in one pass along whole rows or three 1-D passes
+// through tmp2 and tmp1
 template <typename T>
 void launch_prolong(int mf, int mc, int N, const XferTab &t, const T *ec, T *tmp1, T *tmp2,
                     const T *efin, T *efout, cudaStream_t s);
+// Passes fused along whole x-rows (k_rows.cu); rows_fit: the row kernels take
+// the level (m nodes per side, the next level mc) at N columns
+template <typename T>
+bool rows_fit(int m, int mc, int N);
+// sets the dynamic shared-memory limits (call once, outside any stream capture)
+void rows_prepare();
+// out (m x m x mc points) = x-restriction of b - A x
+template <typename T>
+void launch_resid_restrict_x(int m, int mc, int N, const XferTab &t, const T *D, T c, const T *x,
+                             const T *b, T *out, cudaStream_t s);
+// z = the second damped-Jacobi sweep from zero: z1 = wD r, z = S(z1)
+void launch_sweep2(int m, int N, const float *wD, float c, float omw, const float *r, float *z,
+                   cudaStream_t s);
+// out (mc^3) = scaled y- and z-restriction of in (mf x mf x mc)
+template <typename T>
+void launch_restrict_yz(int mf, int mc, int N, const XferTab &t, const T *in, T *out, cudaStream_t s);
+// efout = efin + P ec in one pass; false (nothing launched) when rows of this
+// size do not fit
+template <typename T>
+bool launch_prolong_rows(int mf, int mc, int N, const XferTab &t, const T *ec, const T *efin, T *efout,
+                         cudaStream_t s);
 // z = Ainv r on the coarsest level (Ainv nc x nc, FP64)
 template <typename T>
 void launch_coarse_solve(const GridGeom &g, const double *Ainv, const T *r, T *z,

@@ -7,25 +7,12 @@
 // and every load/store is a 16-byte (or 8-byte) vector access, coalesced
 // across the threads of a warp.  Reductions are per CTA in a fixed order,
 // then over CTAs in a fixed order (deterministic, bit-reproducible).
+#include "grid_common.cuh"
 #include "hq_internal.cuh"
 
 #include <algorithm>
 
 namespace hq {
-
-template <typename T, int V>
-struct alignas(sizeof(T) * V) VT {
-    T v[V];
-};
-
-template <typename T, int V>
-__device__ __forceinline__ VT<T, V> ldv(const T *p) {
-    return *reinterpret_cast<const VT<T, V> *>(p);
-}
-template <typename T, int V>
-__device__ __forceinline__ void stv(T *p, const VT<T, V> &x) {
-    *reinterpret_cast<VT<T, V> *>(p) = x;
-}
 
 GridGeom make_geom(int m, int N, int elem_bytes, int block, int ctas_per_sm) {
     GridGeom g;
@@ -109,99 +96,6 @@ __device__ __forceinline__ void grid_advance(int d, int m, int &i, int &j, int &
             ++kk;
         }
     }
-}
-
-// sum of six neighbours in the order west, east, south, north, below, above;
-// in[k] false: outside the grid (the value loaded for it counts as zero)
-__device__ __forceinline__ float sum6(const float (&x)[6], const bool (&in)[6]) {
-    float a[6];
-#pragma unroll
-    for (int k = 0; k < 6; k++) a[k] = in[k] ? x[k] : 0.f;
-    return ((a[0] + a[1]) + (a[2] + a[3])) + (a[4] + a[5]);
-}
-
-// Six FP64 values summed on the integer pipes.  GB300 retires 0.5 FP64 lanes
-// per clock and scheduler, so the five additions of a 7-point sum hold the
-// FP64 pipe for 280 clocks per warp (measured), more than half of every FP64
-// sweep; the same sum takes about 100 integer-ALU instructions (200 clocks) on
-// another pipe than the products around it.  Measured: the operator at 64^3,
-// 64 columns 272 -> 131 us (FP64 pipe 66%, integer ALU 73% busy), an FP64
-// block PCG at 64^3, 32 columns 10.9 -> 8.1 ms.  Moving the shifts and
-// additions to the FMA pipe as wide multiply-adds was slower (240 against 198
-// clocks per sum).  The terms are aligned to the largest
-// exponent E of the six as 60-bit magnitudes (7 guard bits below the 53 of
-// the largest term), added in 64 bits and rounded once: the error is at most
-// 6 truncations of 2^-59 2^E and one rounding of the result, below that of
-// five rounded additions, whatever their order; the sum is an odd,
-// order-independent function of its terms.  Terms with E outside [64, 2040]
-// (subnormal or near overflow) are scaled by a power of two first; an infinity
-// or a NaN among them takes the plain additions.
-// hi, lo, ex: the words and biased exponents of the six values, E: the largest
-// exponent.
-__device__ __forceinline__ double sum6_aligned(const unsigned (&hi)[6], const unsigned (&lo)[6],
-                                               const unsigned (&ex)[6], unsigned E) {
-    long long s = 0;
-    int neg = 0;   // number of negative terms
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const int sg = (int)hi[k] >> 31;   // all ones for a negative term
-        unsigned mh;   // (hi & 0x000fffff) | 0x00100000 in one instruction
-        asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(mh) : "r"(hi[k]), "r"(0x000fffffu), "r"(0x00100000u));
-        const int vh = (int)__funnelshift_l(lo[k], mh, 7) ^ sg;
-        const unsigned vl = (lo[k] << 7) ^ (unsigned)sg;
-        const long long v = ((long long)vh << 32) | vl;
-        long long w;
-        // one's complement: ~(|v| >> d), one short of -(|v| >> d); shr clamps
-        // shifts of 64 and more (a zero or far smaller term: 0)
-        asm("shr.s64 %0, %1, %2;" : "=l"(w) : "l"(v), "r"(E - ex[k]));
-        s += w;
-        neg -= sg;
-    }
-    s += neg;
-    const int sm = (int)(s >> 32) >> 31;
-    const unsigned long long u = (unsigned long long)((s ^ sm) - sm);
-    // the magnitude's leading bit to bit 62, rounded to the 53 bits 62 .. 10
-    const int lz = __clzll((long long)u);
-    const unsigned long long t = (u << (lz - 1)) + 512ull;
-    const unsigned th = (unsigned)(t >> 32);
-    const unsigned rh = ((th >> 10) + ((E + 3u - (unsigned)lz) << 20)) | ((unsigned)sm & 0x80000000u);
-    return u == 0 ? 0.0 : __hiloint2double((int)rh, (int)__funnelshift_r((unsigned)t, th, 10));
-}
-// a[k] or zero: the terms of the rare exponents
-__device__ __noinline__ double sum6_scaled(double a0, double a1, double a2, double a3, double a4,
-                                           double a5) {
-    double a[6] = {a0, a1, a2, a3, a4, a5};
-    unsigned hi[6], lo[6], ex[6], E = 0;
-#pragma unroll
-    for (int k = 0; k < 6; k++) E = max(E, ((unsigned)__double2hiint(a[k]) << 1) >> 21);
-    if (E == 2047u) return ((a0 + a1) + (a2 + a3)) + (a4 + a5);
-    const bool low = E < 64u;
-    E = 0;
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        a[k] *= low ? 0x1p128 : 0x1p-128;
-        hi[k] = (unsigned)__double2hiint(a[k]);
-        lo[k] = (unsigned)__double2loint(a[k]);
-        ex[k] = (hi[k] << 1) >> 21;
-        E = max(E, ex[k]);
-    }
-    if (E == 0) return 0.0;   // six zeros
-    return sum6_aligned(hi, lo, ex, E) * (low ? 0x1p-128 : 0x1p128);
-}
-__device__ __forceinline__ double sum6(const double (&a)[6], const bool (&in)[6]) {
-    unsigned hi[6], lo[6], ex[6], E = 0;
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        // a term outside the grid gets exponent 0: shifted out whatever its low word
-        hi[k] = in[k] ? (unsigned)__double2hiint(a[k]) : 0u;
-        lo[k] = (unsigned)__double2loint(a[k]);
-        ex[k] = (hi[k] << 1) >> 21;
-        E = max(E, ex[k]);
-    }
-    if (E - 64u > 2040u - 64u)
-        return sum6_scaled(in[0] ? a[0] : 0.0, in[1] ? a[1] : 0.0, in[2] ? a[2] : 0.0,
-                           in[3] ? a[3] : 0.0, in[4] ? a[4] : 0.0, in[5] ? a[5] : 0.0);
-    return sum6_aligned(hi, lo, ex, E);
 }
 
 // Sum of the six neighbours of element e (point (i, j, k) of an m^3 grid) with
@@ -1167,8 +1061,8 @@ __global__ void k_f2d(size_t count, const float *in, double *out) {
 // into the PCG's own passes:
 // k_pcg_xr_mg: x += alpha p, r -= alpha q, partial r.r (all FP64, the
 // geometry of the FP64 level), and the V-cycle's entry: r32 = (float) r and
-// its first damped-Jacobi sweep from zero z32 = wD32 r32 -- the values
-// k_d2f and k_jacobi_first<float> would write.
+// (z32 non-null) its first damped-Jacobi sweep from zero z32 = wD32 r32 -- the
+// values k_d2f and k_jacobi_first<float> would write.
 template <int V>
 __global__ void __launch_bounds__(256) k_pcg_xr_mg(long n, int N, int ppt,
                                                    const double *__restrict__ alpha,
@@ -1203,15 +1097,17 @@ __global__ void __launch_bounds__(256) k_pcg_xr_mg(long n, int N, int ppt,
         }
         stv<double, V>(x + e, xv);
         stv<double, V>(r + e, rv);
-        const float w = wD32[p];
-        VT<float, V> rf, zf;
+        VT<float, V> rf;
 #pragma unroll
-        for (int v = 0; v < V; v++) {
-            rf.v[v] = (float)rv.v[v];
-            zf.v[v] = w * rf.v[v];
-        }
+        for (int v = 0; v < V; v++) rf.v[v] = (float)rv.v[v];
         stv<float, V>(r32 + e, rf);
-        stv<float, V>(z32 + e, zf);
+        if (z32) {
+            const float w = wD32[p];
+            VT<float, V> zf;
+#pragma unroll
+            for (int v = 0; v < V; v++) zf.v[v] = w * rf.v[v];
+            stv<float, V>(z32 + e, zf);
+        }
     }
     block_col_reduce<V, double>(acc, red, part, N, col, cv);
 }
@@ -1541,23 +1437,22 @@ void launch_xfer_tables(int mf, int mc, const XferTab &t, cudaStream_t s) {
                                                            t.pw, t.pwf));
 }
 
-// rc = ((mc+1)/(mf+1))^3 (Rz Ry Rx) rf : x pass (mf,mf,mf)->(mf,mf,mc),
-// y pass ->(mf,mc,mc), z pass (scaled) ->(mc,mc,mc)
+// rc = ((mc+1)/(mf+1))^3 (Rz Ry Rx) rf : x pass (mf,mf,mf)->(mf,mf,mc), then y
+// and z (scaled) ->(mc,mc,mc)
 template <typename T>
-void launch_restrict(int mf, int mc, int N, const XferTab &t, const T *rf, T *tmp1, T *tmp2,
-                     T *rc, cudaStream_t s) {
-    const double q = (double)(mc + 1) / (double)(mf + 1);
+void launch_restrict(int mf, int mc, int N, const XferTab &t, const T *rf, T *tmp1, T *rc,
+                     cudaStream_t s) {
     axis_pass<T, XFER_RTAPS>(mf, mf, mc, mf, 0, N, t.ridx, t.rw, t.rwf, T(1), rf, nullptr, tmp1, s);
-    axis_pass<T, XFER_RTAPS>(mf, mc, mc, mf, 1, N, t.ridx, t.rw, t.rwf, T(1), tmp1, nullptr, tmp2, s);
-    axis_pass<T, XFER_RTAPS>(mc, mc, mc, mf, 2, N, t.ridx, t.rw, t.rwf, (T)(q * q * q), tmp2,
-                             nullptr, rc, s);
+    launch_restrict_yz<T>(mf, mc, N, t, tmp1, rc, s);
 }
 
-// ef_out = ef_in + (Pz Py Px) ec : z pass (mc,mc,mc)->(mf,mc,mc), y pass
-// ->(mf,mf,mc), x pass with the add ->(mf,mf,mf)
+// ef_out = ef_in + (Pz Py Px) ec : whole rows in one pass where they fit, else
+// z pass (mc,mc,mc)->(mf,mc,mc), y pass ->(mf,mf,mc), x pass with the add
+// ->(mf,mf,mf)
 template <typename T>
 void launch_prolong(int mf, int mc, int N, const XferTab &t, const T *ec, T *tmp1, T *tmp2,
                     const T *efin, T *efout, cudaStream_t s) {
+    if (launch_prolong_rows<T>(mf, mc, N, t, ec, efin, efout, s)) return;
     axis_pass<T, 2>(mf, mc, mc, mc, 2, N, t.pidx, t.pw, t.pwf, T(1), ec, nullptr, tmp2, s);
     axis_pass<T, 2>(mf, mf, mc, mc, 1, N, t.pidx, t.pw, t.pwf, T(1), tmp2, nullptr, tmp1, s);
     axis_pass<T, 2>(mf, mf, mf, mc, 0, N, t.pidx, t.pw, t.pwf, T(1), tmp1, efin, efout, s);
@@ -1681,7 +1576,7 @@ void launch_scale(size_t count, const double *factor, T *x, cudaStream_t s) {
                                          cudaStream_t);                                      \
     template void launch_jacobi_rt<T>(const GridGeom &, const T *, T, const T *, const T *,   \
                                       const T *, T *, double *, cudaStream_t);               \
-    template void launch_restrict<T>(int, int, int, const XferTab &, const T *, T *, T *, T *, \
+    template void launch_restrict<T>(int, int, int, const XferTab &, const T *, T *, T *,      \
                                      cudaStream_t);                                          \
     template void launch_prolong<T>(int, int, int, const XferTab &, const T *, T *, T *,      \
                                     const T *, T *, cudaStream_t);                           \
