@@ -129,7 +129,7 @@ struct hq_ctx {
     double *tpart = nullptr;   // gy x N
     double *G2 = nullptr, *Mw = nullptr, *XY = nullptr, *C = nullptr, *T1 = nullptr;
     double *Shat = nullptr, *Om = nullptr, *Msm = nullptr, *Ksm = nullptr, *Ssm = nullptr;
-    double *Lm = nullptr, *Cm = nullptr, *Ym = nullptr, *Cv = nullptr, *Cv2 = nullptr;
+    double *Lm = nullptr, *Cm = nullptr, *Ym = nullptr, *Cv = nullptr;
     double *eigwork = nullptr, *evals = nullptr, *mu = nullptr, *lam_p = nullptr;
     double *lam_r = nullptr, *resn = nullptr, *scal = nullptr, *signwork = nullptr;
     int *status = nullptr;
@@ -487,9 +487,7 @@ size_t carve(hq_ctx *x, const hq_config *c, char *base) {
     double *Cm = cv.take<double>(sizeof(double) * N2);
     double *Ym = cv.take<double>(sizeof(double) * N2);
     double *Cvv = cv.take<double>(sizeof(double) * N2);
-    double *Cv2 = cv.take<double>(sizeof(double) * N2);
-    const size_t P2 = (size_t)((N + 1) & ~1) * ((N + 1) & ~1);
-    double *eigwork = cv.take<double>(sizeof(double) * 2 * P2);
+    double *eigwork = cv.take<double>(sizeof(double) * sym_eig_work_doubles(N));
     double *evals = cv.take<double>(sizeof(double) * N);
     double *mu = cv.take<double>(sizeof(double) * N);
     double *lam_p = cv.take<double>(sizeof(double) * N);
@@ -530,7 +528,7 @@ size_t carve(hq_ctx *x, const hq_config *c, char *base) {
         x->pRw = pRw;
         x->G2 = G2; x->Mw = Mw; x->XY = XY; x->C = Cc; x->T1 = T1; x->Shat = Shat; x->Om = Om;
         x->Msm = Msm; x->Ksm = Ksm; x->Ssm = Ssm; x->Lm = Lm; x->Cm = Cm; x->Ym = Ym;
-        x->Cv = Cvv; x->Cv2 = Cv2; x->eigwork = eigwork; x->evals = evals; x->mu = mu;
+        x->Cv = Cvv; x->eigwork = eigwork; x->evals = evals; x->mu = mu;
         x->lam_p = lam_p; x->lam_r = lam_r; x->resn = resn; x->scal = scal;
         x->signwork = signwork; x->status = status;
     }
@@ -2008,27 +2006,30 @@ hq_status eigen_impl(hq_ctx *x, double *evals_paper, double *evals_rr, double *e
     Level &v0 = x->lev[0];
     GridGeom g64 = make_geom(x->m, N, 8);
     launch_apply<double>(g64, v0.D, v0.c, U64, x->E2, nullptr, x->st);   // (H + sigma) U
-    GramPlan gk = make_gram_plan(x->n, N, N, false);
+    // <U, (H + sigma) U> is symmetric as <U,U> is: the upper tiles of both
     GramPlan gs = make_gram_plan(x->n, N, N, true);
-    launch_gram<double>(gk, U64, N, nullptr, 0, x->E2, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
+    launch_gram<double>(gs, U64, N, nullptr, 0, x->E2, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
     launch_gram<double>(gs, U64, N, nullptr, 0, U64, N, nullptr, 0, x->h3, x->gpart, x->Ssm, x->st);
     launch_axpy_small(N * N, -x->sigma, x->Ssm, x->Ksm, x->st);   // <U, H U>
     launch_rr_reduce(N, x->Ksm, x->Ssm, x->Lm, x->Cm, x->status, x->st);
     HQ_TRY(sync_status(x, x->status, "Rayleigh-Ritz (Cholesky of <U,U>)"));
     launch_sym_eig(N, x->Cm, x->eigwork, x->lam_r, x->Ym, x->st);
     launch_rr_back(N, x->Lm, x->Ym, x->Cv, x->st);
-    TallPlan tp = make_tall_plan(x->n, N, N, N);
+    TallPlan tp = make_tall_plan(x->n, N, N, 0);
     if (evecs || resid) {
-        double *X = (evecs && evecs_on_device) ? evecs : x->E3;
+        // straight into the caller's block where it suits 16-byte accesses
+        const bool direct = evecs && evecs_on_device && ((uintptr_t)evecs & 15u) == 0;
+        double *X = direct ? evecs : x->E3;
         launch_tall_gemm<double>(tp, U64, x->Cv, nullptr, nullptr, nullptr, X, nullptr, x->st);
         launch_fix_signs<double>(x->n, N, X, x->signwork, x->st);
-        if (evecs && !evecs_on_device)
-            HQ_CUDA(cudaMemcpyAsync(evecs, X, cnt * sizeof(double), cudaMemcpyDeviceToHost, x->st));
+        if (evecs && !direct)
+            HQ_CUDA(cudaMemcpyAsync(evecs, X, cnt * sizeof(double), kind_out(evecs_on_device), x->st));
         if (resid) {
-            launch_scale_cols(N, x->Cv, x->lam_r, x->sigma, x->Cv2, x->st);
-            launch_tall_gemm_colsq<double>(tp, x->E2, x->Cv, U64, x->Cv2, nullptr, nullptr,
-                                           x->tpart, x->st);
-            launch_colsum_sqrt(tp.gy, N, x->tpart, x->h3, x->resn, x->st);
+            // || (H + sigma) u_i - (lambda_i + sigma) u_i || with the operator applied to
+            // the Ritz vectors themselves
+            launch_apply<double>(g64, v0.D, v0.c, X, x->E2, nullptr, x->st);
+            launch_pair_resid(g64, x->lam_r, x->sigma, X, x->E2, x->part, x->st);
+            launch_colsum_sqrt(g64.gy, N, x->part, x->h3, x->resn, x->st);
             HQ_CUDA(cudaMemcpyAsync(resid, x->resn, sizeof(double) * N, cudaMemcpyDeviceToHost, x->st));
         }
     }
@@ -2286,16 +2287,16 @@ hq_status rayleigh_ritz_vectors(hq_ctx *x) {
     double *U64 = (double *)x->U;
     Level &v0 = x->lev[0];
     launch_apply<double>(v0.g, v0.D, v0.c, U64, x->E2, nullptr, x->st);   // (H + sigma) U
-    GramPlan gk = make_gram_plan(x->n, N, N, false);
+    // <U, (H + sigma) U> is symmetric as <U,U> is: the upper tiles of both
     GramPlan gs = make_gram_plan(x->n, N, N, true);
-    launch_gram<double>(gk, U64, N, nullptr, 0, x->E2, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
+    launch_gram<double>(gs, U64, N, nullptr, 0, x->E2, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
     launch_gram<double>(gs, U64, N, nullptr, 0, U64, N, nullptr, 0, x->h3, x->gpart, x->Ssm, x->st);
     launch_axpy_small(N * N, -x->sigma, x->Ssm, x->Ksm, x->st);   // <U, H U>
     launch_rr_reduce(N, x->Ksm, x->Ssm, x->Lm, x->Cm, x->status, x->st);
     HQ_TRY(sync_status(x, x->status, "Rayleigh-Ritz (Cholesky of <U,U>)"));
     launch_sym_eig(N, x->Cm, x->eigwork, x->lam_r, x->Ym, x->st);
     launch_rr_back(N, x->Lm, x->Ym, x->Cv, x->st);
-    TallPlan tp = make_tall_plan(x->n, N, N, N);
+    TallPlan tp = make_tall_plan(x->n, N, N, 0);
     launch_tall_gemm<double>(tp, U64, x->Cv, nullptr, nullptr, nullptr, (double *)x->Uh, nullptr,
                              x->st);
     launch_fix_signs<double>(x->n, N, (double *)x->Uh, x->signwork, x->st);
@@ -2346,15 +2347,10 @@ hq_status refine_impl(hq_ctx *x, int rounds, double rtol, int maxit, double *res
     HQ_TRY(copy_blk<double>(x, (double *)x->U, u, cnt));
     if (resid) {
         // ||H u_i - theta_i u_i|| of the final Ritz pairs
-        launch_add_scalar(N, x->lam_r, x->sigma, x->mu, x->st);
         launch_apply<double>(v.g, v.D, v.c, u, b, nullptr, x->st);
-        launch_shift_cols(n, N, x->mu, u, b, x->st);
-        GramPlan gp = make_gram_plan(n, N, N, true);
-        launch_gram<double>(gp, b, N, nullptr, 0, b, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
-        std::vector<double> K((size_t)N * N);
-        HQ_CUDA(cudaMemcpyAsync(K.data(), x->Ksm, sizeof(double) * N * N, cudaMemcpyDeviceToHost, x->st));
-        HQ_CUDA(cudaStreamSynchronize(x->st));
-        for (int i = 0; i < N; i++) resid[i] = std::sqrt(std::max(0.0, K[(size_t)i * N + i]));
+        launch_pair_resid(v.g, x->lam_r, x->sigma, u, b, x->part, x->st);
+        launch_colsum_sqrt(v.g.gy, N, x->part, x->h3, x->resn, x->st);
+        HQ_CUDA(cudaMemcpyAsync(resid, x->resn, sizeof(double) * N, cudaMemcpyDeviceToHost, x->st));
     }
     HQ_CUDA(cudaStreamSynchronize(x->st));
     return check_launch(x);
@@ -2665,6 +2661,7 @@ hq_status hq_init(const hq_config *cfg, void *d_workspace, size_t bytes, void *c
     hq::vcoarse_prepare();
     hq::rows_prepare();
     hq::lu32_prepare();
+    hq::sym_eig_prepare();
     if (x->ozimg || x->ozgram) hq::oz_prepare();
     if (e != cudaSuccess) {
         delete x;

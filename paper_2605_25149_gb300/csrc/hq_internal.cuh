@@ -165,6 +165,9 @@ bool launch_prolong_rows(int mf, int mc, int N, const XferTab &t, const T *ec, c
 template <typename T>
 void launch_coarse_solve(const GridGeom &g, const double *Ainv, const T *r, T *z,
                          cudaStream_t s);
+// partials (g.gy x N) of |y - (lam + add) x|^2 per column (FP64)
+void launch_pair_resid(const GridGeom &g, const double *lam, double add, const double *x,
+                       const double *y, double *part, cudaStream_t s);
 // partial of x.y per column
 template <typename T>
 void launch_dot(const GridGeom &g, const T *x, const T *y, double *part, cudaStream_t s);
@@ -370,23 +373,16 @@ struct TallPlan {
     long n;
     int ncol, k1, k2;
     int gx, gy;
+    int edge;   // columns per tile (<= 64)
 };
 TallPlan make_tall_plan(long n, int ncol, int k1, int k2);
 template <typename T>
 void launch_tall_gemm(const TallPlan &p, const T *A1, const double *M1, const T *A2,
                       const double *M2, const T *Cin, T *Out, double *part_sq,
                       cudaStream_t s);
-// same with per-column partial sums of squares (gy x ncol)
-template <typename T>
-void launch_tall_gemm_colsq(const TallPlan &p, const T *A1, const double *M1, const T *A2,
-                            const double *M2, const T *Cin, T *Out, double *part_sq,
-                            cudaStream_t s);
 // dst (rows x cols, ld ldd) = alpha * src (ld lds)
 void launch_extract(int rows, int cols, double alpha, const double *src, int lds, double *dst,
                     int ldd, cudaStream_t s);
-// out[i][j] = -Cv[i][j] * (lam[j] + add)   (N x N)
-void launch_scale_cols(int N, const double *Cv, const double *lam, double add, double *out,
-                       cudaStream_t s);
 // out[0] = w * sum(part[0..np)); out[1] = ||A - I||_F for N x N A (nullable)
 void launch_monitor_finish(int np, const double *part, double w, int N, const double *A,
                            double *out, cudaStream_t s);
@@ -446,7 +442,11 @@ void launch_corrector_matrix(int N, const double *Shat, const double *tau_dev, d
 void launch_add_diag(int N, double *A, double v, cudaStream_t s);
 // out = alpha * in  (count values)
 void launch_dscale(int count, double alpha, const double *in, double *out, cudaStream_t s);
-// symmetric eigen (cyclic Jacobi, one CTA): ascending evals, evecs columns (N x N)
+// symmetric eigen (cyclic Jacobi): ascending evals, evecs columns (N x N, nullable);
+// work: sym_eig_work_doubles(N) doubles.  sym_eig_prepare: shared-memory limits
+// (call once, outside any stream capture)
+size_t sym_eig_work_doubles(int N);
+void sym_eig_prepare();
 void launch_sym_eig(int N, const double *A, double *work, double *evals, double *evecs,
                     cudaStream_t s);
 // Rayleigh-Ritz reduction: given K (N x N, symmetrised inside) and S (SPD),

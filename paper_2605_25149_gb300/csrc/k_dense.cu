@@ -144,19 +144,29 @@ __global__ void __launch_bounds__(256) k_gram_partial(GramPlan P, const T *A1, i
             if (!diag || i <= j) dst[(ty + 16 * i) * E + tx + 16 * j] = (double)acc[i][j];
 }
 
-// one thread per tile entry (grid: tiles x entry blocks), chunks summed in order
-__global__ void k_gram_reduce(GramPlan P, const double *partials, double w, double *out) {
-    const int tile = blockIdx.x, E = (P.edge + 15) / 16 * 16;
+// CTA = 32 tile entries x 8 threads, each summing an eighth of the chunks in
+// order, then the eighths in order (one thread per entry: 94 us at 64^3 points,
+// 64 columns, 304 chunks; this 21 us)
+__global__ void __launch_bounds__(256) k_gram_reduce(GramPlan P, const double *partials, double w,
+                                                     double *out) {
+    __shared__ double red[8][33];
+    const int tile = blockIdx.x, E = (P.edge + 15) / 16 * 16, g = threadIdx.y;
     int ta, tb;
     tile_of(tile, P.tiles_a, P.sym, ta, tb);
-    const int e = blockIdx.y * blockDim.x + threadIdx.x;
-    if (e >= E * E) return;
+    const int e = blockIdx.y * 32 + threadIdx.x;   // E * E is a multiple of 256
     const int la = e / E, lb = e % E;
-    const bool diag = P.sym && ta == tb;
-    if (diag && la > lb) return;   // its mirror entry's thread writes it
     const int a = ta * P.edge + la, b = tb * P.edge + lb;
-    if (la >= P.edge || lb >= P.edge || a >= P.na || b >= P.nb) return;
-    double s = ordered_sum(partials + (size_t)tile * E * E + e, P.chunks, (size_t)P.ntiles * E * E);
+    // below the diagonal: its mirror entry's thread writes it
+    const bool ok = !(P.sym && ta == tb && la > lb) && la < P.edge && lb < P.edge && a < P.na && b < P.nb;
+    const int per = (P.chunks + 7) / 8, c0 = min(P.chunks, g * per), c1 = min(P.chunks, c0 + per);
+    const size_t stride = (size_t)P.ntiles * E * E;
+    red[g][threadIdx.x] =
+        ok ? ordered_sum(partials + (size_t)tile * E * E + e + c0 * stride, c1 - c0, stride) : 0.0;
+    __syncthreads();
+    if (g != 0 || !ok) return;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) s += red[k][threadIdx.x];
     s *= w;
     out[(size_t)a * P.nb + b] = s;
     if (P.sym && a != b) out[(size_t)b * P.nb + a] = s;
@@ -175,12 +185,12 @@ void launch_gram(const GramPlan &p, const T *A1, int na1, const T *A2, int na2, 
     else if (R == 2) go(k_gram_partial<T, 2>);
     else if (R == 3) go(k_gram_partial<T, 3>);
     else go(k_gram_partial<T, 4>);
-    HQ_LAUNCH(HQ_K_GRAM, k_gram_reduce<<<dim3(p.ntiles, (256 * R * R + 255) / 256), 256, 0, s>>>(
+    HQ_LAUNCH(HQ_K_GRAM, k_gram_reduce<<<dim3(p.ntiles, 8 * R * R), dim3(32, 8), 0, s>>>(
                              p, partials, w, out));
 }
 
 // ---------------------------------------------------------------------------
-// Tall GEMM: Out = A1 M1 + A2 M2 + Cin (64 x 64 output tiles)
+// Tall GEMM: Out = A1 M1 + A2 M2 + Cin (tiles of 64 points x at most 64 columns)
 // ---------------------------------------------------------------------------
 constexpr int TBP = 64, TBN = 64, TKC = 16;
 
@@ -192,67 +202,85 @@ TallPlan make_tall_plan(long n, int ncol, int k1, int k2) {
     p.k2 = k2;
     p.gx = (ncol + TBN - 1) / TBN;
     p.gy = (int)((n + TBP - 1) / TBP);
+    p.edge = (ncol + p.gx - 1) / p.gx;
     return p;
 }
 
-template <typename T>
+// 16 x 16 threads of 4 points x R columns; R the smallest of 1 .. 4 that covers
+// the plan's columns per tile (the FP64 pipe bounds the kernel, a 64-column
+// tile for 32 columns did twice the work).  The next K slice's loads are issued
+// before the products of this one.  Every output is summed over K in order.
+template <typename T, int R>
 __global__ void __launch_bounds__(256) k_tall_gemm(TallPlan P, const T *A1, const double *M1,
                                                    const T *A2, const double *M2, const T *Cin,
-                                                   T *Out, double *part_sq, int colwise) {
+                                                   T *Out, double *part_sq) {
+    constexpr int E = 16 * R;
     __shared__ T As[TBP][TKC + 1];
     __shared__ T Ms[TKC][TBN + 1];
     __shared__ double red[256];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const long p0 = (long)blockIdx.y * TBP;
-    const int c0 = blockIdx.x * TBN;
-    T acc[4][4];
+    const int c0 = blockIdx.x * P.edge;
+    const int s1 = (P.k1 + TKC - 1) / TKC, s2 = A2 ? (P.k2 + TKC - 1) / TKC : 0;   // K slices
+    T acc[4][R];
 #pragma unroll
     for (int i = 0; i < 4; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = T(0);
-    for (int pass = 0; pass < 2; pass++) {
-        const T *A = pass == 0 ? A1 : A2;
-        const double *M = pass == 0 ? M1 : M2;
-        const int K = pass == 0 ? P.k1 : P.k2;
-        if (A == nullptr || K == 0) continue;
-        for (int k0 = 0; k0 < K; k0 += TKC) {
-            for (int idx = threadIdx.x; idx < TBP * TKC; idx += 256) {
-                int r = idx / TKC, kk = idx % TKC;
-                long p = p0 + r;
-                As[r][kk] = (p < P.n && k0 + kk < K) ? A[(size_t)p * K + k0 + kk] : T(0);
-            }
-            for (int idx = threadIdx.x; idx < TKC * TBN; idx += 256) {
-                int kk = idx / TBN, c = idx % TBN;
-                Ms[kk][c] = (k0 + kk < K && c0 + c < P.ncol)
-                                ? (T)M[(size_t)(k0 + kk) * P.ncol + c0 + c]
-                                : T(0);
-            }
-            __syncthreads();
+        for (int j = 0; j < R; j++) acc[i][j] = T(0);
+    T va[TBP * TKC / 256], vm[TKC * E / 256];
+    auto load = [&](int sl) {
+        const T *A = sl < s1 ? A1 : A2;
+        const double *M = sl < s1 ? M1 : M2;
+        const int K = sl < s1 ? P.k1 : P.k2, k0 = (sl < s1 ? sl : sl - s1) * TKC;
 #pragma unroll
-            for (int kk = 0; kk < TKC; kk++) {
-                T a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; i++) a[i] = As[ty + 16 * i][kk];
-#pragma unroll
-                for (int j = 0; j < 4; j++) b[j] = Ms[kk][tx + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-#pragma unroll
-                    for (int j = 0; j < 4; j++) acc[i][j] += a[i] * b[j];
-            }
-            __syncthreads();
+        for (int u = 0; u < TBP * TKC / 256; u++) {
+            const int idx = threadIdx.x + 256 * u, r = idx / TKC, kk = idx % TKC;
+            const long p = p0 + r;
+            va[u] = (p < P.n && k0 + kk < K) ? A[(size_t)p * K + k0 + kk] : T(0);
         }
+#pragma unroll
+        for (int u = 0; u < TKC * E / 256; u++) {
+            const int idx = threadIdx.x + 256 * u, kk = idx / E, c = idx % E;
+            vm[u] = (k0 + kk < K && c0 + c < P.ncol) ? (T)M[(size_t)(k0 + kk) * P.ncol + c0 + c] : T(0);
+        }
+    };
+    load(0);
+    for (int sl = 0; sl < s1 + s2; sl++) {
+#pragma unroll
+        for (int u = 0; u < TBP * TKC / 256; u++) {
+            const int idx = threadIdx.x + 256 * u;
+            As[idx / TKC][idx % TKC] = va[u];
+        }
+#pragma unroll
+        for (int u = 0; u < TKC * E / 256; u++) {
+            const int idx = threadIdx.x + 256 * u;
+            Ms[idx / E][idx % E] = vm[u];
+        }
+        __syncthreads();
+        if (sl + 1 < s1 + s2) load(sl + 1);
+#pragma unroll
+        for (int kk = 0; kk < TKC; kk++) {
+            T a[4], b[R];
+#pragma unroll
+            for (int i = 0; i < 4; i++) a[i] = As[ty + 16 * i][kk];
+#pragma unroll
+            for (int j = 0; j < R; j++) b[j] = Ms[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < R; j++) acc[i][j] += a[i] * b[j];
+        }
+        __syncthreads();
     }
     double sq = 0.0;
-    double sqc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         long p = p0 + ty + 16 * i;
         if (p >= P.n) continue;
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int c = c0 + tx + 16 * j;
-            if (c >= P.ncol) continue;
+        for (int j = 0; j < R; j++) {
+            const int cl = tx + 16 * j, c = c0 + cl;
+            if (cl >= P.edge || c >= P.ncol) continue;
             size_t e = (size_t)p * P.ncol + c;
             T v = acc[i][j];
             if (Cin) v = Cin[e] + v;
@@ -260,33 +288,17 @@ __global__ void __launch_bounds__(256) k_tall_gemm(TallPlan P, const T *A1, cons
             if (part_sq) {
                 double dv = (double)v;
                 sq += dv * dv;
-                sqc[j] += dv * dv;
             }
         }
     }
     if (part_sq) {
-        if (!colwise) {
-            red[threadIdx.x] = sq;
+        red[threadIdx.x] = sq;
+        __syncthreads();
+        for (int w = 128; w > 0; w >>= 1) {
+            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
             __syncthreads();
-            for (int w = 128; w > 0; w >>= 1) {
-                if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-                __syncthreads();
-            }
-            if (threadIdx.x == 0) part_sq[(size_t)blockIdx.y * P.gx + blockIdx.x] = red[0];
-        } else {
-            // per column: reduce over ty (16 rows of threads) in order
-            for (int j = 0; j < 4; j++) {
-                red[threadIdx.x] = sqc[j];
-                __syncthreads();
-                if (ty == 0) {
-                    double s = 0.0;
-                    for (int y = 0; y < 16; y++) s += red[y * 16 + tx];
-                    int c = c0 + tx + 16 * j;
-                    if (c < P.ncol) part_sq[(size_t)blockIdx.y * P.ncol + c] = s;
-                }
-                __syncthreads();
-            }
         }
+        if (threadIdx.x == 0) part_sq[(size_t)blockIdx.y * P.gx + blockIdx.x] = red[0];
     }
 }
 
@@ -294,13 +306,15 @@ template <typename T>
 void launch_tall_gemm(const TallPlan &p, const T *A1, const double *M1, const T *A2,
                       const double *M2, const T *Cin, T *Out, double *part_sq,
                       cudaStream_t s) {
-    HQ_LAUNCH(HQ_K_BLOCKGEMM, k_tall_gemm<T><<<dim3(p.gx, p.gy), 256, 0, s>>>(p, A1, M1, A2, M2, Cin, Out, part_sq, 0));
-}
-template <typename T>
-void launch_tall_gemm_colsq(const TallPlan &p, const T *A1, const double *M1, const T *A2,
-                            const double *M2, const T *Cin, T *Out, double *part_sq,
-                            cudaStream_t s) {
-    HQ_LAUNCH(HQ_K_BLOCKGEMM, k_tall_gemm<T><<<dim3(p.gx, p.gy), 256, 0, s>>>(p, A1, M1, A2, M2, Cin, Out, part_sq, 1));
+    const dim3 grid(p.gx, p.gy);
+    const int R = (p.edge + 15) / 16;
+    auto go = [&](auto kernel) {
+        HQ_LAUNCH(HQ_K_BLOCKGEMM, kernel<<<grid, 256, 0, s>>>(p, A1, M1, A2, M2, Cin, Out, part_sq));
+    };
+    if (R == 1) go(k_tall_gemm<T, 1>);
+    else if (R == 2) go(k_tall_gemm<T, 2>);
+    else if (R == 3) go(k_tall_gemm<T, 3>);
+    else go(k_tall_gemm<T, 4>);
 }
 
 __global__ void k_sum_sqrt(int np, const double *part, double w, double *out) {
@@ -1447,9 +1461,11 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
                 double aip = A[(size_t)i * P + p], aiq = A[(size_t)i * P + q];
                 A[(size_t)i * P + p] = c * aip - sv * aiq;
                 A[(size_t)i * P + q] = sv * aip + c * aiq;
-                double vip = Vv[(size_t)i * P + p], viq = Vv[(size_t)i * P + q];
-                Vv[(size_t)i * P + p] = c * vip - sv * viq;
-                Vv[(size_t)i * P + q] = sv * vip + c * viq;
+                if (evecs) {
+                    double vip = Vv[(size_t)i * P + p], viq = Vv[(size_t)i * P + q];
+                    Vv[(size_t)i * P + p] = c * vip - sv * viq;
+                    Vv[(size_t)i * P + q] = sv * vip + c * viq;
+                }
             }
             __syncthreads();
             for (int k = tid; k < P / 2; k += T) {
@@ -1475,8 +1491,279 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
     }
 }
 
+// The same eigenproblem for N <= SE_MAX in three parts, since one SM's FP64
+// rate (about 2.3 lanes per clock) bounds cyclic Jacobi: an FP64 sweep of N = 64
+// with vectors takes 0.27 ms in shared memory and eight or nine are needed.
+//  1. FP32 Jacobi of A scaled by a power of two (k_sym_eig_sm<float>): V0, whose
+//     columns diagonalise A to 1e-6 of its norm (its rounding floor is near 4e-7);
+//  2. V1 = V0 (15/8 I - 10/8 G + 3/8 G^2), G = V0^T V0: orthogonal to FP64
+//     rounding (the step cubes V0's 1e-6), and A' = V1^T A V1 in FP64 on many CTAs;
+//  3. FP64 Jacobi of A' continuing V1 (k_sym_eig_sm<double>): the off-diagonal
+//     starts at 1e-6, so two or three sweeps meet the criterion of k_sym_eig.
+// A non-finite V0 is replaced by I.  The result is FP64's: part 3 is a complete
+// FP64 Jacobi with the tolerance of k_sym_eig whatever V0 was.
+// Measured, N = 64: 7 ms in one FP64 launch before; now 0.6 + 0.08 + 0.66 ms (0.08 ms
+// for part 1 where A is nearly diagonal, as in every refinement round but the first).
+constexpr int SE_MAX = 112;
+constexpr int SE_THREADS = 1024;
+constexpr int SE_BLK = (SE_MAX / 2 * (SE_MAX / 2 - 1) / 2 + SE_THREADS - 1) / SE_THREADS;
+
+// One-CTA cyclic Jacobi in shared memory, round-robin pairs, the rotations of a
+// round applied to the 2 x 2 blocks of all pairs of pairs at once (each block
+// once, its mirror image written with it).  The tangent of each rotation is
+// formed in FP32 (an inexact angle leaves 1e-7 of the element, which later
+// sweeps remove), its cosine from that tangent to the working precision, so the
+// rotations are orthogonal to rounding.  Elements at or below `skip` are left.
+template <typename T>
+__device__ void jacobi_sweeps(int P, int N, T *A, T *V, T *cs, T *sn, int *pp, int *qq, T *red, T tol,
+                              T skip, int max_sweeps) {
+    const int tid = threadIdx.x, LD = P + 1, H = P / 2;
+    const int blocks = H * (H - 1) / 2;   // at most SE_BLK per thread
+    // blocks of different pairs: (k, k + d mod H), decoded once
+    int bk[SE_BLK], bl[SE_BLK];
+#pragma unroll
+    for (int u = 0; u < SE_BLK; u++) {
+        const int idx = tid + u * SE_THREADS;
+        bk[u] = -1;
+        bl[u] = 0;
+        if (idx < blocks) {
+            const int d = idx / H + 1;
+            bk[u] = idx - (d - 1) * H;
+            bl[u] = bk[u] + d < H ? bk[u] + d : bk[u] + d - H;
+        }
+    }
+    const int warp = tid >> 5, lane = tid & 31;
+    for (int sweep = 0; sweep < max_sweeps; sweep++) {
+        T off = T(0);
+        for (int idx = tid; idx < P * P; idx += SE_THREADS) {
+            const int i = idx / P, j = idx - i * P;
+            if (i < j) off += A[i * LD + j] * A[i * LD + j];
+        }
+        red[tid] = off;
+        __syncthreads();
+        for (int w = SE_THREADS / 2; w > 0; w >>= 1) {
+            if (tid < w) red[tid] += red[tid + w];
+            __syncthreads();
+        }
+        off = red[0];
+        __syncthreads();
+        if (sqrt(off) <= tol || off == T(0)) break;
+        for (int r = 0; r < P - 1; r++) {
+            if (tid < H) {
+                int a = P - 1, b = r;
+                if (tid > 0) {
+                    a = r + tid;
+                    if (a >= P - 1) a -= P - 1;
+                    b = r - tid;
+                    if (b < 0) b += P - 1;
+                }
+                const int p = min(a, b), q = max(a, b);
+                pp[tid] = p;
+                qq[tid] = q;
+                T c = T(1), sv = T(0);
+                const T apq = A[p * LD + q];
+                if (fabs(apq) > skip) {
+                    const float x = (float)(A[q * LD + q] - A[p * LD + p]), y = 2.f * (float)apq;
+                    const float t = (x >= 0.f ? y : -y) / (fabsf(x) + sqrtf(x * x + y * y));
+                    const T u = T(1) + (T)t * (T)t;
+                    c = (T)rsqrtf((float)u);
+                    c = c * (T(1.5) - T(0.5) * u * c * c);
+                    if (sizeof(T) == 8) c = c * (T(1.5) - T(0.5) * u * c * c);
+                    sv = (T)t * c;
+                }
+                cs[tid] = c;
+                sn[tid] = sv;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int b = 0; b < SE_BLK; b++) {
+                const int k = bk[b], l = bl[b];
+                if (k < 0) continue;
+                const T ck = cs[k], sk = sn[k], cl = cs[l], sl = sn[l];
+                if (sk == T(0) && sl == T(0)) continue;
+                const int p = pp[k], q = qq[k], u = pp[l], w = qq[l];
+                const T a11 = A[p * LD + u], a12 = A[p * LD + w], a21 = A[q * LD + u], a22 = A[q * LD + w];
+                const T b11 = ck * a11 - sk * a21, b12 = ck * a12 - sk * a22;
+                const T b21 = sk * a11 + ck * a21, b22 = sk * a12 + ck * a22;
+                const T n11 = cl * b11 - sl * b12, n12 = sl * b11 + cl * b12;
+                const T n21 = cl * b21 - sl * b22, n22 = sl * b21 + cl * b22;
+                A[p * LD + u] = A[u * LD + p] = n11;
+                A[p * LD + w] = A[w * LD + p] = n12;
+                A[q * LD + u] = A[u * LD + q] = n21;
+                A[q * LD + w] = A[w * LD + q] = n22;
+            }
+            if (tid >= SE_THREADS - H) {
+                const int k = tid - (SE_THREADS - H);
+                const T c = cs[k], sv = sn[k];
+                if (sv != T(0)) {
+                    const int p = pp[k], q = qq[k];
+                    const T app = A[p * LD + p], aqq = A[q * LD + q], apq = A[p * LD + q];
+                    const T b11 = c * app - sv * apq, b12 = c * apq - sv * aqq;
+                    const T b21 = sv * app + c * apq, b22 = sv * apq + c * aqq;
+                    A[p * LD + p] = c * b11 - sv * b12;
+                    A[q * LD + q] = sv * b21 + c * b22;
+                    A[p * LD + q] = A[q * LD + p] = sv * b11 + c * b12;
+                }
+            }
+            if (V)
+                for (int k = warp; k < H; k += SE_THREADS / 32) {
+                    const T c = cs[k], sv = sn[k];
+                    if (sv == T(0)) continue;
+                    T *vp = V + pp[k], *vq = V + qq[k];
+                    for (int i = lane; i < N; i += 32) {
+                        const T a = vp[i * LD], b = vq[i * LD];
+                        vp[i * LD] = c * a - sv * b;
+                        vq[i * LD] = sv * a + c * b;
+                    }
+                }
+            __syncthreads();
+        }
+    }
+}
+
+size_t sym_eig_sm_bytes(int N, size_t esz, bool vec) {
+    const size_t P = (N + 1) & ~1, LD = P + 1;
+    return esz * (P * LD + (vec ? N * LD : 0) + P + SE_THREADS) + sizeof(int) * P + 16;
+}
+
+// T = float: Vout = V0 (N x N FP64, columns), As = sym(Ain) scaled by the power of
+// two scale[0] (N x N).  T = double: Ain is A' (scaled), Vin = V1 (nullable: no
+// vectors); evals ascending, divided by scale[0], evecs in their order.
+template <typename T>
+__global__ void __launch_bounds__(SE_THREADS) k_sym_eig_sm(int N, const double *Ain, const double *Vin,
+                                                           double *Vout, double *As, double *scale,
+                                                           double *evals, double *evecs) {
+    extern __shared__ double se_smem[];
+    const int P = (N + 1) & ~1, LD = P + 1, tid = threadIdx.x;
+    constexpr bool F32 = sizeof(T) == 4;
+    T *A = reinterpret_cast<T *>(se_smem), *V = nullptr, *cs = A + P * LD;
+    if (F32 || Vin) {
+        V = cs;
+        cs += N * LD;
+    }
+    T *sn = cs + P / 2, *red = sn + P / 2;
+    int *pp = reinterpret_cast<int *>(red + SE_THREADS), *qq = pp + P / 2;
+    __shared__ double big_sh[32];
+    double sc = 1.0;
+    if (F32) {
+        // power of two bringing the largest entry to [1/2, 1)
+        double big = 0.0;
+        for (int idx = tid; idx < N * N; idx += SE_THREADS) big = fmax(big, fabs(Ain[idx]));
+        for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+        if ((tid & 31) == 0) big_sh[tid >> 5] = big;
+        __syncthreads();
+        for (int w = 0; w < 32; w++) big = fmax(big, big_sh[w]);
+        int e = 0;
+        if (big > 0.0 && isfinite(big)) {
+            frexp(big, &e);
+            e = max(-1000, min(1000, e));
+        }
+        sc = ldexp(1.0, -e);
+        if (tid == 0) scale[0] = sc;
+    }
+    for (int idx = tid; idx < P * P; idx += SE_THREADS) {
+        const int i = idx / P, j = idx - i * P;
+        double a = 0.0;
+        if (i < N && j < N) {
+            a = 0.5 * (Ain[(size_t)i * N + j] * sc + Ain[(size_t)j * N + i] * sc);
+            if (F32) As[(size_t)i * N + j] = a;
+        }
+        A[i * LD + j] = (T)a;
+        if (V && i < N) V[i * LD + j] = F32 ? (i == j ? T(1) : T(0)) : (j < N ? (T)Vin[(size_t)i * N + j] : T(0));
+    }
+    __syncthreads();
+    T fro = T(0);
+    for (int idx = tid; idx < P * P; idx += SE_THREADS) {
+        const int i = idx / P, j = idx - i * P;
+        fro += A[i * LD + j] * A[i * LD + j];
+    }
+    red[tid] = fro;
+    __syncthreads();
+    for (int w = SE_THREADS / 2; w > 0; w >>= 1) {
+        if (tid < w) red[tid] += red[tid + w];
+        __syncthreads();
+    }
+    fro = sqrt(red[0]);
+    __syncthreads();
+    // skipped elements together stay below the tolerance: P^2/2 of them at most
+    const T tol = (F32 ? T(1e-6) : T(1e-15)) * fro;
+    jacobi_sweeps<T>(P, N, A, V, cs, sn, pp, qq, red, tol, tol / (T)(2 * P), F32 ? 12 : 100);
+    if (F32) {
+        __shared__ int bad;
+        if (tid == 0) bad = 0;
+        __syncthreads();
+        for (int idx = tid; idx < N * N; idx += SE_THREADS)
+            if (!isfinite((float)V[(idx / N) * LD + idx % N])) bad = 1;
+        __syncthreads();
+        for (int idx = tid; idx < N * N; idx += SE_THREADS) {
+            const int i = idx / N, j = idx - i * N;
+            Vout[idx] = bad ? (i == j ? 1.0 : 0.0) : (double)V[i * LD + j];
+        }
+        return;
+    }
+    const double back = 1.0 / scale[0];
+    for (int i = tid; i < N; i += SE_THREADS) {
+        const double di = (double)A[i * LD + i];
+        int rank = 0;
+        for (int j = 0; j < N; j++) {
+            const double dj = (double)A[j * LD + j];
+            if (dj < di || (dj == di && j < i)) rank++;
+        }
+        evals[rank] = di * back;
+        if (evecs)
+            for (int k = 0; k < N; k++) evecs[(size_t)k * N + rank] = (double)V[k * LD + i];
+    }
+}
+
+// M = 15/8 I - 10/8 G + 3/8 G^2 (N x N)
+__global__ void k_ortho_poly(int N, const double *G, double *M) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= N * N) return;
+    const int i = e / N, j = e - i * N;
+    double s = 0.0;
+    for (int k0 = 0; k0 < N; k0 += 8) {
+        double a[8], b[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            a[u] = k0 + u < N ? G[(size_t)i * N + k0 + u] : 0.0;
+            b[u] = k0 + u < N ? G[(size_t)(k0 + u) * N + j] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; u++) s += a[u] * b[u];
+    }
+    M[e] = (i == j ? 1.875 : 0.0) - 1.25 * G[e] + 0.375 * s;
+}
+
+void sym_eig_prepare() {
+    cudaFuncSetAttribute(k_sym_eig_sm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sym_eig_sm_bytes(SE_MAX, 4, true));
+    cudaFuncSetAttribute(k_sym_eig_sm<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sym_eig_sm_bytes(SE_MAX, 8, true));
+}
+
+size_t sym_eig_work_doubles(int N) {
+    const size_t P2 = (size_t)((N + 1) & ~1) * ((N + 1) & ~1);
+    return N <= SE_MAX ? 5 * (size_t)N * N + 1 : 2 * P2;
+}
+
 void launch_sym_eig(int N, const double *A, double *work, double *evals, double *evecs,
                     cudaStream_t s) {
+    if (N <= SE_MAX) {
+        const size_t NN = (size_t)N * N;
+        double *V = work, *G = work + NN, *M = work + 2 * NN, *V1 = work + 3 * NN, *As = work + 4 * NN,
+               *scale = work + 5 * NN;
+        HQ_LAUNCH(HQ_K_SMALL, k_sym_eig_sm<float><<<1, SE_THREADS, sym_eig_sm_bytes(N, 4, true), s>>>(
+                                  N, A, nullptr, V, As, scale, nullptr, nullptr));
+        launch_small_gemm(N, N, N, 1.0, V, N, true, V, N, false, 0.0, G, N, s);
+        HQ_LAUNCH(HQ_K_SMALL, k_ortho_poly<<<(unsigned)((NN + 127) / 128), 128, 0, s>>>(N, G, M));
+        launch_small_gemm(N, N, N, 1.0, V, N, false, M, N, false, 0.0, V1, N, s);
+        launch_small_gemm(N, N, N, 1.0, As, N, false, V1, N, false, 0.0, G, N, s);
+        launch_small_gemm(N, N, N, 1.0, V1, N, true, G, N, false, 0.0, M, N, s);
+        HQ_LAUNCH(HQ_K_SMALL,
+                  k_sym_eig_sm<double><<<1, SE_THREADS, sym_eig_sm_bytes(N, 8, evecs != nullptr), s>>>(
+                      N, M, evecs ? V1 : nullptr, nullptr, nullptr, scale, evals, evecs));
+        return;
+    }
     int P = (N + 1) & ~1;
     size_t shm = sizeof(double) * (P + 1024) + sizeof(int) * (P + 2) + 16;
     HQ_LAUNCH(HQ_K_SMALL, k_sym_eig<<<1, 1024, shm, s>>>(N, A, work, evals, evecs));
@@ -1814,17 +2101,23 @@ void launch_chol_solve(int N, const double *A, int lda, const double *B, int ldb
     HQ_LAUNCH(HQ_K_SMALL, k_chol_solve<<<1, 1024, 0, s>>>(N, A, lda, B, ldb, L, X, status));
 }
 
-__global__ void k_rr_back(int N, const double *L, const double *Y, double *Cv) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < N; e += gridDim.x * blockDim.x) {
-        for (int i = N - 1; i >= 0; i--) {
-            double s = Y[(size_t)i * N + e];
-            for (int k = i + 1; k < N; k++) s -= L[(size_t)k * N + i] * Cv[(size_t)k * N + e];
-            Cv[(size_t)i * N + e] = s / L[(size_t)i * N + i];
-        }
+// c = L^{-T} y, one warp per column (x in shared memory, each row's dot product
+// split over the lanes; the thread-per-column form took 240 us at N = 64, this 86 us)
+__global__ void __launch_bounds__(32) k_rr_back(int N, const double *L, const double *Y, double *Cv) {
+    extern __shared__ double bx[];
+    const int e = blockIdx.x, lane = threadIdx.x;
+    for (int i = N - 1; i >= 0; i--) {
+        double part = 0.0;
+        for (int k = i + 1 + lane; k < N; k += 32) part += L[(size_t)k * N + i] * bx[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane == 0) bx[i] = (Y[(size_t)i * N + e] - part) / L[(size_t)i * N + i];
+        __syncwarp();
     }
+    for (int i = lane; i < N; i += 32) Cv[(size_t)i * N + e] = bx[i];
 }
 void launch_rr_back(int N, const double *L, const double *Y, double *Cv, cudaStream_t s) {
-    HQ_LAUNCH(HQ_K_SMALL, k_rr_back<<<(N + 127) / 128, 128, 0, s>>>(N, L, Y, Cv));
+    HQ_LAUNCH(HQ_K_SMALL, k_rr_back<<<N, 32, sizeof(double) * N, s>>>(N, L, Y, Cv));
 }
 
 __global__ void k_inv_sqrt_first(const double *ev, double *out) { out[0] = 1.0 / sqrt(ev[0]); }
@@ -1879,30 +2172,38 @@ __global__ void k_sign_pass1(long n, int N, const T *U, long rows, double *work)
         work[((size_t)blockIdx.y * N + c) * 2 + 1] = (double)bi[0];
     }
 }
+// Pass 2: per column, the sign of its largest entry over the slabs (in order)
 template <typename T>
-__global__ void k_sign_pass2(long n, int N, T *U, int gy, const double *work) {
-    const int c = blockIdx.x;
-    __shared__ double sgn;
-    if (threadIdx.x == 0) {
-        double best = -1.0;
-        long idx = -1;
-        for (int y = 0; y < gy; y++) {
-            double v = work[((size_t)y * N + c) * 2];
-            long i = (long)work[((size_t)y * N + c) * 2 + 1];
-            if (v > best) { best = v; idx = i; }
-        }
-        sgn = (idx >= 0 && U[(size_t)idx * N + c] < T(0)) ? -1.0 : 1.0;
+__global__ void k_sign_pick(int N, const T *U, int gy, double *work) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= N) return;
+    double best = -1.0;
+    long idx = -1;
+    for (int y = 0; y < gy; y++) {
+        const double v = work[((size_t)y * N + c) * 2];
+        const long i = (long)work[((size_t)y * N + c) * 2 + 1];
+        if (v > best) { best = v; idx = i; }
     }
-    __syncthreads();
-    if (sgn > 0) return;
-    for (long p = threadIdx.x; p < n; p += blockDim.x) U[(size_t)p * N + c] = -U[(size_t)p * N + c];
+    work[(size_t)c * 2] = (idx >= 0 && U[(size_t)idx * N + c] < T(0)) ? -1.0 : 1.0;
+}
+// Pass 3: the columns of negative sign, all points at once (whole rows: one CTA
+// per column reads 8 bytes of every row, 711 us at 64^3, 64 columns; this: 45 us)
+template <typename T>
+__global__ void __launch_bounds__(256) k_sign_flip(long n, int N, T *U, const double *work) {
+    for (int c = threadIdx.x; c < N; c += 32) {
+        if (work[(size_t)c * 2] > 0.0) continue;
+        for (long p = (long)blockIdx.x * 8 + threadIdx.y; p < n; p += (long)gridDim.x * 8)
+            U[(size_t)p * N + c] = -U[(size_t)p * N + c];
+    }
 }
 template <typename T>
 void launch_fix_signs(long n, int N, T *U, double *work, cudaStream_t s) {
     int gy = (int)std::min<long>(64, (n + 1023) / 1024);
     long rows = (n + gy - 1) / gy;
     HQ_LAUNCH(HQ_K_SMALL, k_sign_pass1<T><<<dim3(N, gy), 256, 0, s>>>(n, N, U, rows, work));
-    HQ_LAUNCH(HQ_K_SMALL, k_sign_pass2<T><<<N, 256, 0, s>>>(n, N, U, gy, work));
+    HQ_LAUNCH(HQ_K_SMALL, k_sign_pick<T><<<(N + 63) / 64, 64, 0, s>>>(N, U, gy, work));
+    const int blocks = (int)std::min<long>((n + 7) / 8, 152 * 8);
+    HQ_LAUNCH(HQ_K_SMALL, k_sign_flip<T><<<blocks, dim3(32, 8), 0, s>>>(n, N, U, work));
 }
 
 __global__ void k_extract(int rows, int cols, double alpha, const double *src, int lds,
@@ -1920,21 +2221,6 @@ void launch_extract(int rows, int cols, double alpha, const double *src, int lds
                                                                 ldd));
 }
 
-__global__ void k_scale_cols(int N, const double *Cv, const double *lam, double add,
-                             double *out) {
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N * N;
-         idx += gridDim.x * blockDim.x) {
-        int j = idx % N;
-        out[idx] = -Cv[idx] * (lam[j] + add);
-    }
-}
-void launch_scale_cols(int N, const double *Cv, const double *lam, double add, double *out,
-                       cudaStream_t s) {
-    HQ_LAUNCH(HQ_K_SMALL, k_scale_cols<<<std::min((N * N + 255) / 256, 1024), 256, 0, s>>>(N, Cv, lam, add, out));
-}
-
-// out[0] = w * sum of all np*ncol partials (fixed order); out[1] = ||A - I||_F
-// of the N x N matrix A (nullable)
 __global__ void k_monitor_finish(int np, const double *part, double w, int N, const double *A,
                                  double *out) {
     __shared__ double red[256];
@@ -1976,9 +2262,6 @@ void launch_monitor_finish(int np, const double *part, double w, int N, const do
     template void launch_tall_gemm<T>(const TallPlan &, const T *, const double *, const T *, \
                                       const double *, const T *, T *, double *,              \
                                       cudaStream_t);                                         \
-    template void launch_tall_gemm_colsq<T>(const TallPlan &, const T *, const double *,      \
-                                            const T *, const double *, const T *, T *,        \
-                                            double *, cudaStream_t);                         \
     template void launch_fix_signs<T>(long, int, T *, double *, cudaStream_t);
 
 HQ_DINST(double)

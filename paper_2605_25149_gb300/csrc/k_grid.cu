@@ -458,6 +458,37 @@ __global__ void __launch_bounds__(256) k_widen_dot(long n, int N, int ppt,
     if (part) block_col_reduce<V, double>(acc, red, part, N, col, cv);
 }
 
+// partials of |y - (lam + add) x|^2 per column: residual norms of the pairs
+// (lam, x) from y = (H + sigma) x
+template <int V>
+__global__ void __launch_bounds__(256) k_pair_resid(long n, int N, int ppt, const double *__restrict__ lam,
+                                                    double add, const double *__restrict__ x,
+                                                    const double *__restrict__ y, double *part) {
+    __shared__ double red[1024];
+    const int TY = blockDim.y;
+    const int col = (blockIdx.x * blockDim.x + threadIdx.x) * V;
+    const bool cv = col < N;
+    double acc[V], s[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        acc[v] = 0.0;
+        s[v] = cv ? lam[col + v] + add : 0.0;
+    }
+    const long base = (long)blockIdx.y * TY * ppt;
+    for (int k = 0; k < ppt; k++) {
+        long p = base + (long)k * TY + threadIdx.y;
+        if (!cv || p >= n) continue;
+        size_t e = (size_t)p * N + col;
+        VT<double, V> xv = ldv<double, V>(x + e), yv = ldv<double, V>(y + e);
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            const double d = yv.v[v] - s[v] * xv.v[v];
+            acc[v] += d * d;
+        }
+    }
+    block_col_reduce<V, double>(acc, red, part, N, col, cv);
+}
+
 template <typename T, int V>
 __global__ void __launch_bounds__(256) k_jacobi_first(long n, int N, int ppt,
                                                       const T *__restrict__ wD,
@@ -1486,6 +1517,17 @@ static void run_widen_dot(const GridGeom &g, const float *z32, const double *r, 
 void launch_widen_dot(const GridGeom &g, const float *z32, const double *r, double *z,
                       double *part, cudaStream_t s) {
     HQ_VEC_DISPATCH(double, g, run_widen_dot, g, z32, r, z, part, s);
+}
+
+template <typename T, int V>
+static void run_pair_resid(const GridGeom &g, const double *lam, double add, const double *x,
+                           const double *y, double *part, cudaStream_t s) {
+    HQ_LAUNCH_W(HQ_K_VECTOR, (double)g.n * g.N,
+                k_pair_resid<V><<<grd(g), blk(g), 0, s>>>(g.n, g.N, g.ppt, lam, add, x, y, part));
+}
+void launch_pair_resid(const GridGeom &g, const double *lam, double add, const double *x,
+                       const double *y, double *part, cudaStream_t s) {
+    HQ_VEC_DISPATCH(double, g, run_pair_resid, g, lam, add, x, y, part, s);
 }
 
 template <typename T>

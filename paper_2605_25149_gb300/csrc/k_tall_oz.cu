@@ -17,8 +17,9 @@
 // per term).  The epilogue combines D_2..D_9 in 64-bit fixed point, converts
 // once to FP64, applies 2^(e_p + f_c), adds Cin and optionally sums squares.
 //
-// CTA = 128 points x 64 output columns, all K; per 64-wide K chunk the 256
-// threads convert the FP64 rows into 8 digit planes (K-major, 128-byte
+// CTA = 128 points x 64 output columns, all K; per 64-wide K chunk the 512
+// threads (256 hid less of the latencies: 355 against 321 us at 64^3, K = 64)
+// convert the FP64 rows into 8 digit planes (K-major, 128-byte
 // swizzle) while bulk copies bring the 8 digit planes of the small matrix
 // (prepared once per call by k_oz_split); one thread issues 36 MMAs per K
 // step of 16.  TMEM: 8 accumulators x 64 columns = 512 columns.  The output
@@ -38,7 +39,8 @@ constexpr int OZ_NT = 64;                 // output columns per CTA
 constexpr int OZ_KC = 64;                 // K per chunk: 128 bytes of bf16 per row
 constexpr int OZ_S = 8;                   // digits per value
 constexpr int OZ_BITS = 7;                // bits per digit
-constexpr int OZ_THREADS = 256;           // 8 warps: warp w reads TMEM lanes 32 (w % 4)..
+constexpr int OZ_THREADS = 512;           // 16 warps: warp w reads TMEM lanes 32 (w % 4)..
+constexpr int OZ_EC = OZ_NT / (OZ_THREADS / 128);   // output columns per thread (16)
 constexpr int OZ_APLANE = OZ_M * 128;     // one digit plane of the point rows: 16 KB
 constexpr int OZ_BPLANE = OZ_NT * 128;    // one digit plane of the small matrix: 8 KB
 constexpr int OZ_SMEM = OZ_S * (OZ_APLANE + OZ_BPLANE) + 1024;
@@ -344,34 +346,34 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         }
         __syncthreads();
         // epilogue: thread = one point row (TMEM lane 32 (warp % 4) + lane) and
-        // one half of the 64 output columns (warp / 4)
+        // OZ_EC of the 64 output columns (warp / 4)
         const int r = (warp & 3) * 32 + lane;
         const long p = r0 + r;
         const int em = erow[r];
         {
-            const int cb = (warp >> 2) * 32;
+            const int cb = (warp >> 2) * OZ_EC;
             // sum_t D_t 2^(-7(t-2)) as a 64-bit fixed-point integer with 40
             // fraction bits (|D_2| < 2^21: no overflow; the two smallest
             // scales lose at most 2^-39), so the FP64 pipe sees one
             // conversion per output instead of a Horner chain
-            long long acc[32];
+            long long acc[OZ_EC];
 #pragma unroll
-            for (int j = 0; j < 32; j++) acc[j] = 0;
+            for (int j = 0; j < OZ_EC; j++) acc[j] = 0;
 #pragma unroll
             for (int t = 2; t <= OZ_S + 1; t++) {
-                float v[32];
-                tmem_ld32<32>(tmem + ((uint32_t)((warp & 3) * 32) << 16) +
+                float v[OZ_EC];
+                tmem_ld32<OZ_EC>(tmem + ((uint32_t)((warp & 3) * 32) << 16) +
                                   (uint32_t)((t - 2) * OZ_NT + cb), v);
                 const int sh = OZ_FRAC - OZ_BITS * (t - 2);
 #pragma unroll
-                for (int j = 0; j < 32; j++) {
+                for (int j = 0; j < OZ_EC; j++) {
                     const long long d = (long long)__float2int_rn(v[j]);
                     acc[j] += sh >= 0 ? (d << sh) : (d >> (-sh));
                 }
             }
             if (p < n) {
 #pragma unroll
-            for (int j = 0; j < 32; j++) {
+            for (int j = 0; j < OZ_EC; j++) {
                 const int c = ct * OZ_NT + cb + j;
                 if (c >= ncol) continue;
                 const int fc = fexp[c];
@@ -681,16 +683,26 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
                      : "memory");
 }
 
-// out[i][j] = w * sum over chunks (in order) of the chunk partials, for the
-// columns of the ctiles tiles from tile ct0 on (the others are not written)
-__global__ void k_oz_gram_reduce(int na, int ct0, int ctiles, int chunks, const double *partials,
-                                 double w, double *out) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= na * na) return;
+// out[i][j] = w * sum over chunks of the chunk partials, for the columns of the
+// ctiles tiles from tile ct0 on (the others are not written).  CTA = 32
+// entries x 8 threads, each summing an eighth of the chunks in order, then the
+// eighths in order (one thread per entry waited for 152 dependent loads: 42 us
+// at na = 128; see k_gram_reduce)
+__global__ void __launch_bounds__(256) k_oz_gram_reduce(int na, int ct0, int ctiles, int chunks,
+                                                        const double *partials, double w, double *out) {
+    __shared__ double red[8][33];
+    const int e = blockIdx.x * 32 + threadIdx.x, g = threadIdx.y;
     const int i = e / na, j = e % na, ct = j / OZ_NT - ct0, jl = j % OZ_NT;
-    if (ct < 0) return;
-    const double s = ordered_sum(partials + ((size_t)ct * OZ_M + i) * OZ_NT + jl, chunks,
-                                 (size_t)ctiles * OZ_M * OZ_NT);
+    const bool ok = e < na * na && ct >= 0;
+    const int per = (chunks + 7) / 8, c0 = min(chunks, g * per), c1 = min(chunks, c0 + per);
+    const size_t stride = (size_t)ctiles * OZ_M * OZ_NT;
+    red[g][threadIdx.x] =
+        ok ? ordered_sum(partials + ((size_t)ct * OZ_M + i) * OZ_NT + jl + c0 * stride, c1 - c0, stride) : 0.0;
+    __syncthreads();
+    if (g != 0 || !ok) return;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) s += red[k][threadIdx.x];
     out[e] = w * s;
 }
 
@@ -757,7 +769,7 @@ void launch_gram_oz(long n, const double *X1, int n1, const double *X2, int n2, 
     HQ_LAUNCH(HQ_K_GRAM, k_gram_oz<<<dim3(nt, g.chunks), OZ_GTHREADS, OZ_GSMEM, s>>>(
                              n, n1, n2, g.chunk_rows, ct0, X1, n2 ? X2 : nullptr, colexp, partials,
                              status));
-    HQ_LAUNCH(HQ_K_GRAM, k_oz_gram_reduce<<<(na * na + 255) / 256, 256, 0, s>>>(
+    HQ_LAUNCH(HQ_K_GRAM, k_oz_gram_reduce<<<(na * na + 31) / 32, dim3(32, 8), 0, s>>>(
                              na, ct0, nt, g.chunks, partials, w, out));
 }
 
