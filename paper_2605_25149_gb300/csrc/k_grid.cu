@@ -735,41 +735,52 @@ __global__ void __launch_bounds__(256) k_finalize(int mode, int N, int gy, const
     red[0][warp][lane] = s;
     red[1][warp][lane] = s2;
     __syncthreads();
-    if (warp == 0) {
-        double a = 0.0, b = 0.0;
+    if (R == 1) {
+        // one chunk: its sums are the result (no arrival to wait for: a third of
+        // the latency of the small problems' reductions)
+        if (warp != 0 || col >= N) return;
+        s = s2 = 0.0;
         for (int w = 0; w < 8; w++) {
-            a += red[0][w][lane];
-            b += red[1][w][lane];
+            s += red[0][w][lane];
+            s2 += red[1][w][lane];
         }
-        if (col < N) {
-            sc.fpart[(size_t)blockIdx.y * N + col] = a;
-            sc.fpart[(size_t)(R + blockIdx.y) * N + col] = b;
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(&sc.fcount[blockIdx.x], 1u) == (unsigned)(R - 1));
-    __syncthreads();
-    if (!last || warp != 0) return;
-    __threadfence();
-    if (lane == 0) sc.fcount[blockIdx.x] = 0u;
-    if (col >= N) return;
-    s = 0.0;
-    s2 = 0.0;
-    for (int c0 = 0; c0 < R; c0 += 8) {
-        double a[8], b[8];
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const int c = c0 + u;
-            a[u] = c < R ? __ldcg(&sc.fpart[(size_t)c * N + col]) : 0.0;
-            b[u] = c < R ? __ldcg(&sc.fpart[(size_t)(R + c) * N + col]) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; u++)
-            if (c0 + u < R) {
-                s += a[u];
-                s2 += b[u];
+    } else {
+        if (warp == 0) {
+            double a = 0.0, b = 0.0;
+            for (int w = 0; w < 8; w++) {
+                a += red[0][w][lane];
+                b += red[1][w][lane];
             }
+            if (col < N) {
+                sc.fpart[(size_t)blockIdx.y * N + col] = a;
+                sc.fpart[(size_t)(R + blockIdx.y) * N + col] = b;
+            }
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) last = (atomicAdd(&sc.fcount[blockIdx.x], 1u) == (unsigned)(R - 1));
+        __syncthreads();
+        if (!last || warp != 0) return;
+        __threadfence();
+        if (lane == 0) sc.fcount[blockIdx.x] = 0u;
+        if (col >= N) return;
+        s = 0.0;
+        s2 = 0.0;
+        for (int c0 = 0; c0 < R; c0 += 8) {
+            double a[8], b[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                const int c = c0 + u;
+                a[u] = c < R ? __ldcg(&sc.fpart[(size_t)c * N + col]) : 0.0;
+                b[u] = c < R ? __ldcg(&sc.fpart[(size_t)(R + c) * N + col]) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (c0 + u < R) {
+                    s += a[u];
+                    s2 += b[u];
+                }
+        }
     }
     switch (mode) {
     case FIN_BNORM_RNORM: {

@@ -389,13 +389,17 @@ RowShape row_shape(int len, int N) {
     s.q = (len + s.ty - 1) / s.ty;
     return s;
 }
-// chunks of a march of `len` steps so that about 16 CTAs per SM exist, each
-// of at least four steps (2 to 16 per SM measured: 64^3, 64 columns 320, 301, 294,
-// 299 us per V-cycle, 96^3 925, 871, 854, 834 us, 128^3 within 2%)
+// steps per CTA of a march of `len` steps: about 16 CTAs per SM (2 to 16 per SM
+// measured: 64^3, 64 columns 320, 301, 294, 299 us per V-cycle, 96^3 925, 871, 854,
+// 834 us, 128^3 within 2%) but at least four steps; fewer where even so the CTAs
+// do not fill four per SM (a step waits for its loads, so on small levels the
+// march itself was the time: y/z-restriction of 16^3, 32 columns 16 us)
 int march_chunk(long ctas, int len) {
-    long ch = (152L * 16 + ctas - 1) / ctas;
-    ch = std::max(1L, std::min(ch, (long)std::max(1, len / 4)));
-    return (int)((len + ch - 1) / ch);
+    auto chunk = [&](long target) {
+        const long ch = std::max(1L, std::min((long)len, (target + ctas - 1) / ctas));
+        return (int)((len + ch - 1) / ch);
+    };
+    return std::max(chunk(152L * 16), std::min(4, chunk(152L * 4)));
 }
 template <typename T>
 size_t row_smem_bytes(const RowShape &s, int m, int mc) {
