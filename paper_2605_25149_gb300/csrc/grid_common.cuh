@@ -111,4 +111,14 @@ __device__ __forceinline__ double sum6(const double (&a)[6], const bool (&in)[6]
     return sum6_aligned(hi, lo, ex, E);
 }
 
+// (double) f through integers: a conversion is an FP64-pipe instruction (56
+// clocks per warp, as an FMA), the bit form seven of the integer ALU.  Zeros,
+// subnormals, infinities and NaN take the conversion.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e - 0x00800000u >= 0x7f000000u) return (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                            (int)(u << 29));
+}
+
 }  // namespace hq

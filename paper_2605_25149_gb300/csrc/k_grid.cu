@@ -447,10 +447,13 @@ __global__ void __launch_bounds__(256) k_widen_dot(long n, int N, int ppt,
         long p = base + (long)k * TY + threadIdx.y;
         if (!cv || p >= n) continue;
         size_t e = (size_t)p * N + col;
-        VT<double, V> rv = ldv<double, V>(r + e), o;
+        VT<double, V> rv, o;
+        if (part) rv = ldv<double, V>(r + e);
+        const VT<float, V> zv = ldv<float, V>(z32 + e);
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            o.v[v] = (double)z32[e + v];
+            o.v[v] = widen(zv.v[v]);
+            if (!part) continue;
             acc[v] += rv.v[v] * o.v[v];
         }
         stv<double, V>(z + e, o);
@@ -1188,7 +1191,7 @@ __global__ void __launch_bounds__(256) k_jacobi_dot64(int m, long n, int N, int 
 #pragma unroll
         for (int v = 0; v < V; v++) o.v[v] = omw * zc.v[v] + w * (rv.v[v] + c * sm.v[v]);
 #pragma unroll
-        for (int v = 0; v < V; v++) acc[v] += r8.v[v] * (double)o.v[v];
+        for (int v = 0; v < V; v++) acc[v] += r8.v[v] * widen(o.v[v]);
         stv<float, V>(zout + e, o);
     }
     block_col_reduce<V, double>(acc, red, part, N, col, cv);
@@ -1215,7 +1218,7 @@ __global__ void __launch_bounds__(256) k_pcg_p_mg(long n, int N, int ppt,
         VT<float, V> zv = ldv<float, V>(z32 + e);
         VT<double, V> pv = ldv<double, V>(p_ + e);
 #pragma unroll
-        for (int v = 0; v < V; v++) pv.v[v] = (double)zv.v[v] + bt[v] * pv.v[v];
+        for (int v = 0; v < V; v++) pv.v[v] = widen(zv.v[v]) + bt[v] * pv.v[v];
         stv<double, V>(p_ + e, pv);
     }
 }

@@ -21,8 +21,8 @@
 // threads (256 hid less of the latencies: 355 against 321 us at 64^3, K = 64)
 // convert the FP64 rows into 8 digit planes (K-major, 128-byte
 // swizzle) while bulk copies bring the 8 digit planes of the small matrix
-// (prepared once per call by k_oz_split); one thread issues 36 MMAs per K
-// step of 16.  TMEM: 8 accumulators x 64 columns = 512 columns.  The output
+// (prepared once per call by k_oz_split); one thread issues the 36 digit
+// products of a K step of 16 as 12 MMAs.  TMEM: 8 accumulators x 64 columns = 512 columns.  The output
 // tile is staged in the freed digit planes for whole-row Cin reads and Out
 // writes.  Every wait is bounded.
 #include "hq_internal.cuh"
@@ -107,6 +107,36 @@ __device__ __forceinline__ void oz_digits2(double x0, double x1, int emax, uint3
     }
 }
 
+// sum_t D_t 2^(-7(t-2)), t = 2 .. 9, of 16 columns as 64-bit fixed point with FRAC
+// fraction bits.  Neighbouring digit sums join in 32 bits (128 D_t + D_{t+1}:
+// below 2^31 since |D_t| < 2^24 and only D_2 .. D_8 are shifted, |D_8| < 7 2^21),
+// the four halves in 64: q0 in units 2^-21, q1 in units 2^-49, of which one
+// truncation (below 2^-FRAC) remains.  tm: the thread's lane and first column.
+template <int FRAC>
+__device__ __forceinline__ void oz_combine(uint32_t tm, long long (&acc)[16], bool add) {
+#pragma unroll
+    for (int g = 0; g < 16; g += 8) {
+        long long q0[8];
+        int p[8];
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            float a[8], b[8];
+            tmem_ld8x2(tm + (uint32_t)(2 * h * OZ_NT + g), tm + (uint32_t)((2 * h + 1) * OZ_NT + g), a, b);
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                const int s = __float2int_rn(a[j]) * 128 + __float2int_rn(b[j]);
+                if ((h & 1) == 0) {
+                    p[j] = s;
+                } else {
+                    const long long q = (long long)p[j] * 16384 + s;
+                    if (h == 1) q0[j] = q << (FRAC - 21);
+                    else acc[g + j] = (add ? acc[g + j] : 0ll) + q0[j] + (q >> (49 - FRAC));
+                }
+            }
+        }
+    }
+}
+
 __device__ __forceinline__ double pow2(int e) {
     // 2^e for |e| <= 2000 as a product of two normal powers of two
     const int e1 = e / 2, e2 = e - e1;
@@ -167,12 +197,36 @@ __global__ void __launch_bounds__(256) k_oz_rowexp(long n, int k1, int k2, const
     if (lane == 0) erow[p] = em;
 }
 
+// acc 2^es, rounded to FP64: the leading bit to the implicit one by integer
+// shifts (the conversion of a 64-bit integer is three FP64-pipe instructions,
+// which held that pipe for 10,000 of a tile's 37,000 clocks)
+__device__ __forceinline__ double oz_scaled(long long acc, int es) {
+    const long long sm = acc >> 63;
+    const unsigned long long u = (unsigned long long)((acc ^ sm) - sm);   // < 2^63
+    if (u == 0) return 0.0;
+    const int lz = __clzll((long long)u), ex = 1086 - lz + es;
+    if (ex < 1 || ex > 2045) {   // subnormal or overflowing result
+        const double v = (double)acc;
+        return es >= -1022 && es <= 1023 ? v * __longlong_as_double((long long)(es + 1023) << 52) : v * pow2(es);
+    }
+    const unsigned long long t = (u << (lz - 1)) + 512ull;
+    const unsigned long long bits = (t >> 10) + ((unsigned long long)(ex - 1) << 52);
+    return __longlong_as_double((long long)(bits | ((unsigned long long)sm << 63)));
+}
+
+// Persistent: one CTA per SM strides the tiles (point blocks x column tiles, the
+// column tiles of a point block next to each other); an item's start, its TMEM
+// allocation and its end cost a third of the one-tile-per-CTA form.  Per 64-wide
+// K chunk the digit planes are written in two halves of 32, and the MMAs of the
+// first run while the second is converted.  Measured at 64^3 points, K = 64, 64
+// columns: 334 -> 230 us (with Cin 375 -> 269); of a tile's 35,000 clocks the
+// conversion takes 6,000, the exposed MMAs 7,000, the epilogue 14,000 (removing
+// its arithmetic saves 6,000) and the output rows 3,200.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_tall_oz(long n, int k1, int k2, int ncol, int kchunks, const double *__restrict__ A1,
+    k_tall_oz(long n, int k1, int k2, int ncol, int kchunks, int ctiles, const double *__restrict__ A1,
               const double *__restrict__ A2, const unsigned char *__restrict__ image,
               const int *__restrict__ fexp, const int *__restrict__ erow_g,
-              const double *__restrict__ Cin, double *__restrict__ Out, double *part_sq,
-              int *status) {
+              const double *Cin, double *Out, double *part_sq, int *status) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *planesA = smem;
@@ -180,19 +234,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __shared__ uint64_t mbar, bbar;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int erow[OZ_M];
-    __shared__ int abort_sh, pend_sh, tmem_free_sh;
-    __shared__ double red[OZ_THREADS];
+    __shared__ __align__(16) int fexp_sh[OZ_NT];   // largest exponents of the tile's columns
+    __shared__ int abort_sh, tmem_free_sh;
+    __shared__ double red[OZ_THREADS / 32];
     constexpr uint32_t TCOLS = OZ_S * OZ_NT;   // 512
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long r0 = (long)blockIdx.x * OZ_M;
-    const int ct = blockIdx.y;
     const int K = k1 + k2;
     if (tid == 0) {
         mbar_init(&mbar, 1);
         mbar_init(&bbar, 1);
         abort_sh = 0;
-        pend_sh = 0;
         tmem_free_sh = 1;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -203,205 +255,210 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    auto aval = [&](long p, int k) -> double {
-        return k < k1 ? A1[(size_t)p * k1 + k] : A2[(size_t)p * k2 + (k - k1)];
-    };
-    // row exponents: from k_oz_rowexp when K spans several chunks, else
-    // formed below from the chunk's values (erow_g null)
-    if (erow_g)
-        for (int r = tid; r < OZ_M; r += OZ_THREADS) erow[r] = (r0 + r < n) ? erow_g[r0 + r] : 0;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base_sh;
-    const uint32_t idesc = idesc_bf16(OZ_M, OZ_NT);
+    const long pblocks = (n + OZ_M - 1) / OZ_M, tiles = pblocks * ctiles;
+    unsigned commits = 0, bulks = 0;   // thread 0: completed phases of mbar, bbar
+    int resident = -1;                 // thread 0: (column tile, chunk) in planesB
+    bool copying = false;              // thread 0: a wait for the bulk copies gave up
 
-    for (int ch = 0; ch < kchunks; ch++) {
-        if (ch > 0 && tid == 0) {
-            if (!mbar_wait(&mbar, (unsigned)((ch - 1) & 1))) {
-                abort_sh = 1;
-                pend_sh = (ch - 1) & 1;
-            }
-        }
-        // the chunk's digit planes of the small matrix (prepared by
-        // k_oz_split) arrive by bulk copies while the threads convert A;
-        // the previous chunk's MMAs, which read them, are complete here
-        if (tid == 0 && !abort_sh) {
-            const unsigned char *src = image + (size_t)(ct * kchunks + ch) * OZ_S * OZ_BPLANE;
-            mbar_expect_tx(&bbar, (uint32_t)(OZ_S * OZ_BPLANE));
+    // A values of chunk ch of point block pb: half-warp hw takes rows
+    // warp 8 + 2 q + hw, lane kk of it the pairs k = 32 h + 2 kk, + 1
+    constexpr int RPW = OZ_M / (OZ_THREADS / 32);   // rows per warp (8)
+    const int hw = lane >> 4, kk = lane & 15;
+    double xv[2][RPW / 2][2];
+    auto load = [&](long pb, int ch) {
 #pragma unroll
-            for (int j = 0; j < OZ_S; j++)
-                bulk_g2s(planesB + j * OZ_BPLANE, src + j * OZ_BPLANE, OZ_BPLANE, &bbar);
-        }
-        __syncthreads();
-        if (abort_sh) break;
-        // digit planes of the point rows for K = ch*64 .. ch*64+63: a warp owns
-        // 16 rows, a lane the pair k = 2 lane, 2 lane + 1 of each (one 32-bit
-        // store per plane; a warp's stores fill one 128-byte row); all 32
-        // loads of a batch of 16 rows are issued before converting
-        {
-            constexpr int RPW = OZ_M / (OZ_THREADS / 32);   // rows per warp
-            double xv[RPW][2];
+        for (int h = 0; h < 2; h++)
 #pragma unroll
-            for (int q = 0; q < RPW; q++) {
-                const int r = warp * RPW + q;
-                const long p = r0 + r;
+            for (int q = 0; q < RPW / 2; q++) {
+                const long p = pb * OZ_M + warp * RPW + 2 * q + hw;
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const int kg = ch * OZ_KC + 2 * lane + h;
-                    xv[q][h] = (p < n && kg < K) ? aval(p, kg) : 0.0;
+                for (int e = 0; e < 2; e++) {
+                    const int k = ch * OZ_KC + 32 * h + 2 * kk + e;
+                    double v = 0.0;
+                    if (p < n && k < K) v = k < k1 ? A1[(size_t)p * k1 + k] : A2[(size_t)p * k2 + (k - k1)];
+                    xv[h][q][e] = v;
                 }
             }
+    };
+    if ((long)blockIdx.x < tiles) load((long)blockIdx.x / ctiles, 0);
+
+    for (long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const long pb = tile / ctiles, r0 = pb * OZ_M;
+        const int ct = (int)(tile % ctiles);
+        // row exponents: from k_oz_rowexp when K spans several chunks, else
+        // formed below from the chunk's values (erow_g null)
+        if (erow_g)
+            for (int r = tid; r < OZ_M; r += OZ_THREADS) erow[r] = (r0 + r < n) ? erow_g[r0 + r] : 0;
+        if (tid < OZ_NT) fexp_sh[tid] = ct * OZ_NT + tid < ncol ? fexp[ct * OZ_NT + tid] : 0;
+        for (int ch = 0; ch < kchunks; ch++) {
+            // the planes are free: the MMAs of the previous chunk or tile were
+            // waited for
+            if (ch > 0 && tid == 0 && !mbar_wait(&mbar, (commits++) & 1u)) abort_sh = 1;
+            if (tid == 0 && !abort_sh && resident != ct * kchunks + ch) {
+                // the chunk's digit planes of the small matrix arrive by bulk
+                // copies while the threads convert A
+                const unsigned char *src = image + (size_t)(ct * kchunks + ch) * OZ_S * OZ_BPLANE;
+                mbar_expect_tx(&bbar, (uint32_t)(OZ_S * OZ_BPLANE));
 #pragma unroll
-            for (int q = 0; q < RPW; q++) {
-                const int r = warp * RPW + q;
-                int em;
+                for (int j = 0; j < OZ_S; j++)
+                    bulk_g2s(planesB + j * OZ_BPLANE, src + j * OZ_BPLANE, OZ_BPLANE, &bbar);
+            }
+            __syncthreads();
+            if (abort_sh) break;
+            int em[RPW / 2];
+#pragma unroll
+            for (int q = 0; q < RPW / 2; q++) {
+                const int r = warp * RPW + 2 * q + hw;
                 if (erow_g) {
-                    em = erow[r];
+                    em[q] = erow[r];
                 } else {
-                    em = __reduce_max_sync(0xffffffffu, (unsigned)max(biased_exp(xv[q][0]),
-                                                                      biased_exp(xv[q][1])));
-                    if (lane == 0) erow[r] = em;
+                    em[q] = max(max(biased_exp(xv[0][q][0]), biased_exp(xv[0][q][1])),
+                                max(biased_exp(xv[1][q][0]), biased_exp(xv[1][q][1])));
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1)   // over the row's 16 lanes
+                        em[q] = max(em[q], __shfl_xor_sync(0xffffffffu, em[q], o));
+                    if (kk == 0) erow[r] = em[q];
                 }
-                uint32_t pk[OZ_S];
-                oz_digits2(xv[q][0], xv[q][1], em, pk);
-                const uint32_t off = sw128_offset16(r, 2 * lane);
-#pragma unroll
-                for (int i = 0; i < OZ_S; i++)
-                    *reinterpret_cast<uint32_t *>(planesA + i * OZ_APLANE + off) = pk[i];
             }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0 && !mbar_wait(&bbar, (unsigned)(ch & 1))) {
-            // no MMA of this chunk is issued; the last commit (if any) was
-            // waited for above
-            abort_sh = 1;
-            pend_sh = (ch + 1) & 1;
-        } else if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int ks = 0; ks < OZ_KC / 16; ks++) {
-                const uint32_t ko = ks * 32;
+            for (int h = 0; h < 2; h++) {
 #pragma unroll
-                for (int t = 2; t <= OZ_S + 1; t++) {
-                    const int ilo = t - OZ_S > 1 ? t - OZ_S : 1;
-                    const int ihi = t - 1 < OZ_S ? t - 1 : OZ_S;
-                    for (int i = ilo; i <= ihi; i++) {
-                        const int j = t - i;
-                        const uint64_t da = make_desc_sw128(smem_u32(planesA + (i - 1) * OZ_APLANE) + ko);
-                        const uint64_t db = make_desc_sw128(smem_u32(planesB + (j - 1) * OZ_BPLANE) + ko);
-                        const uint32_t acc = (ch > 0 || ks > 0 || i > ilo) ? 1u : 0u;
-                        mma_bf16(tmem + (uint32_t)((t - 2) * OZ_NT), da, db, idesc, acc);
+                for (int q = 0; q < RPW / 2; q++) {
+                    const int r = warp * RPW + 2 * q + hw;
+                    uint32_t pk[OZ_S];
+                    oz_digits2(xv[h][q][0], xv[h][q][1], em[q], pk);
+                    const uint32_t off = sw128_offset16(r, 32 * h + 2 * kk);
+#pragma unroll
+                    for (int i = 0; i < OZ_S; i++)
+                        *reinterpret_cast<uint32_t *>(planesA + i * OZ_APLANE + off) = pk[i];
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncthreads();
+                if (tid == 0 && !abort_sh) {
+                    if (h == 0 && resident != ct * kchunks + ch) {
+                        if (mbar_wait(&bbar, bulks & 1u)) {
+                            resident = ct * kchunks + ch;
+                            bulks++;
+                        } else {
+                            abort_sh = 1;   // no MMA of this chunk is issued
+                            copying = true;
+                        }
+                    }
+                    if (!abort_sh) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                        for (int ks = 2 * h; ks < 2 * h + 2; ks++) {
+                            // digit i of A times digits j = 1 .. 9 - i of the small
+                            // matrix: their planes follow each other as 64-row
+                            // blocks of one B operand and so do the accumulators
+                            // D_{i+1} .. D_9, so up to four digits make one MMA of
+                            // 256 columns (12 MMAs in place of 36 of 64 columns,
+                            // each of which took 80 clocks, the time A's rows take)
+                            const uint32_t ko = ks * 32;
+#pragma unroll
+                            for (int i = 1; i <= OZ_S; i++) {
+                                const uint64_t da = make_desc_sw128(smem_u32(planesA + (i - 1) * OZ_APLANE) + ko);
+#pragma unroll
+                                for (int j = 1; j <= 9 - i; j += 4) {
+                                    const int cnt = 10 - i - j < 4 ? 10 - i - j : 4;
+                                    const uint64_t db =
+                                        make_desc_sw128(smem_u32(planesB + (j - 1) * OZ_BPLANE) + ko);
+                                    mma_bf16(tmem + (uint32_t)((i + j - 2) * OZ_NT), da, db,
+                                             idesc_bf16(OZ_M, cnt * OZ_NT), (ch > 0 || ks > 0 || i > 1) ? 1u : 0u);
+                                }
+                            }
+                        }
+                        if (h == 1) mma_commit(&mbar);
                     }
                 }
             }
-            mma_commit(&mbar);
+            if (abort_sh) break;   // (set before the barrier of the second half)
+            if (ch + 1 < kchunks) load(pb, ch + 1);
         }
-    }
-    // the tile's rows and columns; Cin's tile is loaded (coalesced: a warp
-    // reads 32 consecutive columns of one row) while the last MMAs run
-    const int ncl = min(OZ_NT, ncol - ct * OZ_NT);
-    const long nrw = min((long)OZ_M, n - r0);
-    constexpr int EPT = OZ_M * OZ_NT / OZ_THREADS;   // tile elements per thread
-    double cpre[EPT];
-    if (Cin) {
+        if (abort_sh) break;
+        // the tile's rows and columns; the next tile's first values and Cin's
+        // tile (coalesced: a warp reads 32 consecutive columns of one row) are
+        // loaded while the last MMAs run
+        if (tile + gridDim.x < tiles) load((tile + gridDim.x) / ctiles, 0);
+        const int ncl = min(OZ_NT, ncol - ct * OZ_NT);
+        const long nrw = min((long)OZ_M, n - r0);
+        constexpr int EPT = OZ_M * OZ_NT / OZ_THREADS;   // tile elements per thread
+        double cpre[EPT];
+        if (Cin) {
 #pragma unroll
-        for (int u = 0; u < EPT; u++) {
-            const int idx = tid + u * OZ_THREADS, rr = idx / OZ_NT, jj = idx % OZ_NT;
-            cpre[u] = (rr < nrw && jj < ncl) ? Cin[(size_t)(r0 + rr) * ncol + ct * OZ_NT + jj]
-                                             : 0.0;
+            for (int u = 0; u < EPT; u++) {
+                const int idx = tid + u * OZ_THREADS, rr = idx / OZ_NT, jj = idx % OZ_NT;
+                cpre[u] = (rr < nrw && jj < ncl) ? Cin[(size_t)(r0 + rr) * ncol + ct * OZ_NT + jj] : 0.0;
+            }
         }
-    }
-    if (!abort_sh && tid == 0) {
-        if (!mbar_wait(&mbar, (unsigned)((kchunks - 1) & 1))) {
-            abort_sh = 1;
-            pend_sh = (kchunks - 1) & 1;
-        }
-    }
-    // after a wait that gave up, the MMAs of the last commit may still be
-    // writing TMEM: one more bounded wait for them before the columns are
-    // released; if they are still running, the columns stay allocated (only
-    // the status word is meaningful after a timeout)
-    if (abort_sh && tid == 0) tmem_free_sh = mbar_wait(&mbar, (unsigned)pend_sh) ? 1 : 0;
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    double sq = 0.0;
-    if (abort_sh) {
-        if (tid == 0) atomicOr(status, ST_TC_TIMEOUT);
-    } else {
+        if (tid == 0 && !mbar_wait(&mbar, (commits++) & 1u)) abort_sh = 1;
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (abort_sh) break;
         // the digit planes are free once the MMAs are done: the output tile is
         // staged there (row stride OZ_SLD doubles: a half-warp's 8-byte
-        // accesses to one column of 16 rows, or to 16 columns of one row,
-        // fall in distinct banks), so Cin is read and Out written in whole
-        // rows
+        // accesses to one column of 16 rows, or to 16 columns of one row, fall
+        // in distinct banks), so Cin is read and Out written in whole rows
         double *stg = reinterpret_cast<double *>(planesA);
+        double sq = 0.0;
         if (Cin) {
 #pragma unroll
             for (int u = 0; u < EPT; u++) {
                 const int idx = tid + u * OZ_THREADS;
                 stg[(idx / OZ_NT) * OZ_SLD + idx % OZ_NT] = cpre[u];
             }
+            __syncthreads();
         }
-        __syncthreads();
-        // epilogue: thread = one point row (TMEM lane 32 (warp % 4) + lane) and
-        // OZ_EC of the 64 output columns (warp / 4)
-        const int r = (warp & 3) * 32 + lane;
-        const long p = r0 + r;
-        const int em = erow[r];
         {
-            const int cb = (warp >> 2) * OZ_EC;
-            // sum_t D_t 2^(-7(t-2)) as a 64-bit fixed-point integer with 40
-            // fraction bits (|D_2| < 2^21: no overflow; the two smallest
-            // scales lose at most 2^-39), so the FP64 pipe sees one
-            // conversion per output instead of a Horner chain
+            // epilogue: thread = one point row (TMEM lane 32 (warp % 4) + lane)
+            // and OZ_EC of the 64 output columns (warp / 4)
+            const int r = (warp & 3) * 32 + lane, cb = (warp >> 2) * OZ_EC;
+            const int em = erow[r];
+            // a 64-bit fixed-point integer with 40 fraction bits (|D_2| < 2^21:
+            // no overflow)
             long long acc[OZ_EC];
+            oz_combine<OZ_FRAC>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cb, acc, false);
+            // the columns' exponents, ahead of the outputs
+            int fc[OZ_EC];
 #pragma unroll
-            for (int j = 0; j < OZ_EC; j++) acc[j] = 0;
-#pragma unroll
-            for (int t = 2; t <= OZ_S + 1; t++) {
-                float v[OZ_EC];
-                tmem_ld32<OZ_EC>(tmem + ((uint32_t)((warp & 3) * 32) << 16) +
-                                  (uint32_t)((t - 2) * OZ_NT + cb), v);
-                const int sh = OZ_FRAC - OZ_BITS * (t - 2);
-#pragma unroll
-                for (int j = 0; j < OZ_EC; j++) {
-                    const long long d = (long long)__float2int_rn(v[j]);
-                    acc[j] += sh >= 0 ? (d << sh) : (d >> (-sh));
-                }
+            for (int j = 0; j < OZ_EC; j += 4) {
+                const int4 f = *reinterpret_cast<const int4 *>(fexp_sh + cb + j);
+                fc[j] = f.x;
+                fc[j + 1] = f.y;
+                fc[j + 2] = f.z;
+                fc[j + 3] = f.w;
             }
-            if (p < n) {
+            double *sl = stg + r * OZ_SLD + cb;
 #pragma unroll
             for (int j = 0; j < OZ_EC; j++) {
-                const int c = ct * OZ_NT + cb + j;
-                if (c >= ncol) continue;
-                const int fc = fexp[c];
-                const int es = (em - 1022) + (fc - 1022) - 2 * OZ_BITS - OZ_FRAC;
-                // the integer converts exactly or rounds once; the scaling by
-                // 2^es is an add to the exponent field when the result stays
-                // normal (one FP64 operation fewer per output), else a multiply
-                const double a = (double)acc[j];
-                const long long ab = __double_as_longlong(a);
-                const int ea = (int)((ab >> 52) & 0x7FF) + es;
-                double o;
-                if (em == OZ_EBAD || fc == OZ_EBAD)
-                    o = __longlong_as_double(0x7FF8000000000000ll);
-                else if (ea - es != 0 && ea >= 1 && ea <= 2046)
-                    o = __longlong_as_double(ab + (long long)es * (1ll << 52));
-                else if (es >= -1022 && es <= 1023)
-                    o = a * __longlong_as_double((long long)(es + 1023) << 52);
-                else
-                    o = a * pow2(es);
-                double *sl = stg + r * OZ_SLD + cb + j;
-                if (Cin) o += *sl;
-                *sl = o;
+                const int es = (em - 1022) + (fc[j] - 1022) - 2 * OZ_BITS - OZ_FRAC;
+                double o = em == OZ_EBAD || fc[j] == OZ_EBAD ? __longlong_as_double(0x7FF8000000000000ll)
+                                                             : oz_scaled(acc[j], es);
+                if (Cin) o += sl[j];
+                sl[j] = o;
+                // points and columns beyond the block: zero digits, o = 0 (+ Cin's 0)
                 if (part_sq) sq = fma(o, o, sq);
             }
-            }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        if (part_sq) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if (lane == 0) red[warp] = sq;
+        }
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (part_sq && tid == 0) {
+            double v = 0.0;
+            for (int w = 0; w < OZ_THREADS / 32; w++) v += red[w];
+            part_sq[(size_t)pb * ctiles + ct] = v;
         }
         if (Out) {
-            __syncthreads();
 #pragma unroll
             for (int u = 0; u < EPT; u++) {
                 const int idx = tid + u * OZ_THREADS, rr = idx / OZ_NT, jj = idx % OZ_NT;
@@ -409,15 +466,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     Out[(size_t)(r0 + rr) * ncol + ct * OZ_NT + jj] = stg[rr * OZ_SLD + jj];
             }
         }
+        __syncthreads();   // the staged tile and erow are read: the next tile may write them
     }
-    if (part_sq) {
-        red[tid] = sq;
-        __syncthreads();
-        for (int k = OZ_THREADS / 2; k > 0; k >>= 1) {
-            if (tid < k) red[tid] += red[tid + k];
-            __syncthreads();
-        }
-        if (tid == 0) part_sq[(size_t)blockIdx.x * gridDim.y + blockIdx.y] = red[0];
+    __syncthreads();
+    if (abort_sh && tid == 0) {
+        atomicOr(status, ST_TC_TIMEOUT);
+        // the MMAs of the last commit may still be writing TMEM, the bulk copies
+        // shared memory: one more bounded wait for them before the columns are
+        // released; if the MMAs are still running, the columns stay allocated
+        // (only the status word is meaningful after a timeout)
+        if (copying) mbar_wait(&bbar, bulks & 1u);
+        if (commits > 0) tmem_free_sh = mbar_wait(&mbar, (commits - 1) & 1u) ? 1 : 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -536,18 +595,7 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
 #pragma unroll
     for (int j = 0; j < 16; j++) facc[j] = 0;
     auto flush = [&]() {
-#pragma unroll
-        for (int t = 2; t <= OZ_S + 1; t++) {
-            float v[16];
-            tmem_ld32<16>(tmem + ((uint32_t)((warp & 3) * 32) << 16) +
-                              (uint32_t)((t - 2) * OZ_NT + gcb), v);
-            const int sh = OZ_GFRAC - OZ_BITS * (t - 2);
-#pragma unroll
-            for (int j = 0; j < 16; j++) {
-                const long long d = (long long)__float2int_rn(v[j]);
-                facc[j] += sh >= 0 ? (d << sh) : (d >> (-sh));
-            }
-        }
+        oz_combine<OZ_GFRAC>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)gcb, facc, true);
     };
     if (warp == OZ_GCONV / 32) {
         if (lane == 0) {
@@ -791,8 +839,8 @@ void launch_tall_oz(long n, const double *A1, int k1, const double *M1, const do
                                       n, k1, k2, A1, k2 ? A2 : nullptr, erow));
     const unsigned gx = (unsigned)((n + OZ_M - 1) / OZ_M);
     HQ_LAUNCH(HQ_K_BLOCKGEMM,
-              k_tall_oz<<<dim3(gx, ctiles), OZ_THREADS, OZ_SMEM, s>>>(
-                  n, k1, k2, ncol, kchunks, A1, k2 ? A2 : nullptr, image, fexp,
+              k_tall_oz<<<(unsigned)std::min(152L, (long)gx * ctiles), OZ_THREADS, OZ_SMEM, s>>>(
+                  n, k1, k2, ncol, kchunks, ctiles, A1, k2 ? A2 : nullptr, image, fexp,
                   kchunks > 1 ? erow : nullptr, Cin, Out,
                   part_sq, status));
 }
