@@ -111,6 +111,23 @@ __device__ __forceinline__ double sum6(const double (&a)[6], const bool (&in)[6]
     return sum6_aligned(hi, lo, ex, E);
 }
 
+// (A x)_p and (b - A x)_p of a point from its neighbour sum, with the roundings
+// spelled out where kernels have to agree bit for bit
+__device__ __forceinline__ double op_value(double d, double x, double c, double s) {
+    return fma(d, x, -(c * s));
+}
+__device__ __forceinline__ float op_value(float d, float x, float c, float s) { return d * x - c * s; }
+__device__ __forceinline__ double resid_value(double b, double d, double x, double c, double s) {
+    return fma(c, s, fma(-d, x, b));
+}
+__device__ __forceinline__ float resid_value(float b, float d, float x, float c, float s) {
+    return (b - d * x) + c * s;
+}
+
+// groups in which the thread rows of a CTA are summed (block_col_reduce): the
+// rows of a group in order, then the groups in order
+__host__ __device__ __forceinline__ int row_groups(int ty) { return ty >= 16 ? 8 : 1; }
+
 // (double) f through integers: a conversion is an FP64-pipe instruction (56
 // clocks per warp, as an FMA), the bit form seven of the integer ALU.  Zeros,
 // subnormals, infinities and NaN take the conversion.

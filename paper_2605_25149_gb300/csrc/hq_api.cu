@@ -997,8 +997,32 @@ PcgGraph *pcg_graph(hq_ctx *x, T *X, double rtol, int maxit) {
     return &pg;
 }
 
+// the whole solve of a small FP64 problem with the FP32 preconditioner runs as
+// one launch (k_pcg_small): where the V-cycle is one launch from level 0 on
+// (HQ_FUSED_COARSE=0 and the z-marching order keep the separate kernels)
+bool pcg_in_one_launch(const hq_ctx *x) {
+    return x->mg32 && x->fuse_l0 == 0 && !x->no_fuse && x->lev[0].g.zch == 0 && x->mg[0].g.zch == 0 &&
+           pcg_small_fits(make_vcoarse(x, 0), x->lev[0].g);
+}
+
 template <typename T>
 hq_status pcg(hq_ctx *x, const T *B, T *X, double rtol, int maxit, int *iters_host) {
+    if constexpr (std::is_same<T, double>::value) {
+        if (pcg_in_one_launch(x)) {
+            Level &l = x->lev[0];
+            launch_pcg_small(make_vcoarse(x, 0), l.g, l.D, l.c, B, X, x->sc, rtol, maxit, nullptr, 0, x->st);
+            int it[2] = {0, 0};   // columns still active, iterations
+            HQ_CUDA(cudaMemcpyAsync(it, x->sc.num_active, sizeof(it), cudaMemcpyDeviceToHost, x->st));
+            if (iters_host)
+                HQ_CUDA(cudaMemcpyAsync(iters_host, x->sc.iters, sizeof(int) * x->N, cudaMemcpyDeviceToHost, x->st));
+            HQ_TRY(sync_status(x, x->sc.status, "inner PCG"));
+            x->stat_solves++;
+            x->stat_iters += it[1];
+            if (it[0] > 0 && maxit > 0 && rtol > 0.0)
+                return fail(x, HQ_ERR_NOT_CONVERGED, "inner PCG reached cg_maxit");
+            return HQ_OK;
+        }
+    }
     Level &v = x->lev[0];
     const GridGeom &g = v.g;
     const int N = x->N;
@@ -1152,6 +1176,14 @@ bool capture_graph_of(cudaStream_t s, cudaGraph_t *g) {
 template <typename T>
 hq_status pcg_device(hq_ctx *x, const T *B, T *X, double rtol, int maxit, StepGraph &sgr,
                      long long *counters) {
+    if constexpr (std::is_same<T, double>::value) {
+        if (pcg_in_one_launch(x)) {
+            Level &l = x->lev[0];
+            launch_pcg_small(make_vcoarse(x, 0), l.g, l.D, l.c, B, X, x->sc, rtol, maxit, counters,
+                             rtol > 0.0 ? 1 : 0, x->st);
+            return HQ_OK;
+        }
+    }
     Level &v = x->lev[0];
     const GridGeom &g = v.g;
     const int N = x->N;

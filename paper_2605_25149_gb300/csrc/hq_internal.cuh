@@ -176,7 +176,7 @@ void launch_dot(const GridGeom &g, const T *x, const T *y, double *part, cudaStr
 // one CTA per column, every level's vectors in shared memory.  Arrays are
 // indexed from l0 (entry 0 = level l0); the last entry is the coarsest level.
 constexpr int VC_MAXLEV = 8;
-constexpr int VC_MAX_SMEM = 200 * 1024;
+constexpr int VC_MAX_SMEM = 226 * 1024;
 struct VCoarse {
     int levels;                       // levels in the launch (>= 2)
     int m[VC_MAXLEV];                 // nodes per side
@@ -204,6 +204,17 @@ void launch_vcoarse(const VCoarse &v, int N, const float *r, float *z, cudaStrea
 size_t vcoarse64_smem_bytes(const VCoarse &v, const GridGeom &g64);
 void launch_vcoarse64(const VCoarse &v, const GridGeom &g64, const double *r64, double *z64,
                       double *part, cudaStream_t s);
+
+// The block PCG X = (H + sigma)^-1 B of an FP64 problem with the FP32
+// preconditioner (v: the V-cycle from level 0, g: the FP64 geometry) in one
+// launch, the solve of the separate kernels bit for bit.  Leaves bnorm, rnorm,
+// iters, active per column, num_active[0] (columns active at maxit) and
+// num_active[1] (iterations of the slowest column), which counters[0]
+// (nullable) receives too; ST_PCG_MAXIT at the cap when check_maxit.
+bool pcg_small_fits(const VCoarse &v, const GridGeom &g);
+void launch_pcg_small(const VCoarse &v, const GridGeom &g, const double *D64, double c64, const double *B,
+                      double *X, const PcgScalars &sc, double rtol, int maxit, long long *counters,
+                      int check_maxit, cudaStream_t s);
 
 // per-column reduction of gy partials + PCG scalar logic
 enum FinMode { FIN_BNORM_RNORM = 0, FIN_ALPHA = 1, FIN_RR = 2, FIN_BETA = 3, FIN_RZ = 4 };

@@ -46,9 +46,9 @@ void enable_zmarch(GridGeom &g) {
 
 // Per-column partial sums: each thread holds acc[V] for its columns; reduce
 // over threadIdx.y in order and store one row of the partial array.  One
-// thread per output (column group, slot) sums the thread rows, so the chains
-// run side by side.  FP64 partials are summed in FP64 (row order as ever);
-// FP32 partials in FP32 and widened once per output (the thread partials
+// thread per output (column group, slot) and row group (row_groups) sums the
+// thread rows, so the chains run side by side.  FP64 partials are summed in
+// FP64; FP32 partials in FP32 and widened once per output (the thread partials
 // are FP32 sums already; widening each one made the reduction an FP64-pipe
 // cost comparable to the sweep itself at GB300's FP64 rate).
 template <int V, typename A>
@@ -57,21 +57,40 @@ __device__ __forceinline__ void block_col_reduce(A (&acc)[V], double *red, doubl
     (void)col;
     (void)cv;
     const int tx = threadIdx.x, ty = threadIdx.y, TX = blockDim.x, TY = blockDim.y;
+    const int tid = ty * TX + tx, T = TX * TY, no = TX * V;
     A *ra = reinterpret_cast<A *>(red);
 #pragma unroll
-    for (int v = 0; v < V; v++) ra[(ty * TX + tx) * V + v] = acc[v];
+    for (int v = 0; v < V; v++) ra[tid * V + v] = acc[v];
     __syncthreads();
-    // TX V outputs over TX TY threads (64-thread CTAs of 32 column groups of
-    // four: two outputs per thread)
+    const int G = row_groups(TY);
+    if (G > 1) {
+        // at most two sums per thread: 8 no <= 2 T for 16 or more thread rows
+        const int rows = (TY + G - 1) / G;
+        A s[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int idx = tid + u * T, g = idx / no, o = idx - g * no;
+            s[u] = A(0);
+            if (idx < no * G)
+                for (int y = g * rows; y < min(TY, (g + 1) * rows); y++) s[u] += ra[y * no + o];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+            if (tid + u * T < no * G) ra[tid + u * T] = s[u];
+        __syncthreads();
+    }
+    // no outputs over T threads (64-thread CTAs of 32 column groups of four:
+    // two outputs per thread)
+    const int rows = G > 1 ? G : TY;
     if (part)
-        for (int o = ty * TX + tx; o < TX * V; o += TX * TY) {
-            const int cx = o / V, vv = o - cx * V;
-            const int c = (blockIdx.x * TX + cx) * V;   // the column group's first column
+        for (int o = tid; o < no; o += T) {
+            const int c = blockIdx.x * no + o;   // the output's column
             if (c < N) {
                 A s = A(0);
 #pragma unroll 4
-                for (int y = 0; y < TY; y++) s += ra[(y * TX + cx) * V + vv];
-                part[(size_t)blockIdx.y * N + c + vv] = (double)s;
+                for (int y = 0; y < rows; y++) s += ra[y * no + o];
+                part[(size_t)blockIdx.y * N + c] = (double)s;
             }
         }
     __syncthreads();
@@ -157,7 +176,7 @@ __global__ void __launch_bounds__(256) k_stencil(int m, long n, int N, int ppt,
         if (MODE == 1) bb = ldv<T, V>(b + e);
 #pragma unroll
         for (int v = 0; v < V; v++)
-            o.v[v] = MODE == 1 ? (bb.v[v] - d * xc.v[v]) + c * s.v[v] : d * xc.v[v] - c * s.v[v];
+            o.v[v] = MODE == 1 ? resid_value(bb.v[v], d, xc.v[v], c, s.v[v]) : op_value(d, xc.v[v], c, s.v[v]);
         if (MODE == 1) {
 #pragma unroll
             for (int v = 0; v < V; v++) {
@@ -402,8 +421,8 @@ __global__ void __launch_bounds__(256) k_stencil_zm(int m, int N, int nseg, int 
             for (int v = 0; v < V; v++) {
                 const T a[6] = {a0.v[v], a1.v[v], a2.v[v], a3.v[v], xprev.v[v], xnext.v[v]};
                 const T sum = sum6(a, in);
-                o.v[v] = MODE == 1 ? (bb.v[v] - d * xcur.v[v]) + c * sum
-                                   : d * xcur.v[v] - c * sum;
+                o.v[v] = MODE == 1 ? resid_value(bb.v[v], d, xcur.v[v], c, sum)
+                                   : op_value(d, xcur.v[v], c, sum);
             }
             if (MODE == 1) {
 #pragma unroll
