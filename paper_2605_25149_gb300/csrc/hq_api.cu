@@ -2154,18 +2154,15 @@ hq_status level_check(hq_ctx *x, int level, bool need_next) {
 // the number of points (~3e-11 of |u| |y| at 64^3 for localised u), which let
 // the Krylov space of a 1e-11 adjoint solve leak into span(u) and stall.  A
 // looser solve (the refinement's inexact Newton steps) takes the tensor-core
-// Gram of [u y] (rows 0..N-1, columns N..2N-1 of the 2N x 2N result, in the
-// predictor scratch, unused outside a step).
+// Gram (its scratch: that of the 2N columns of a step).
 hq_status project(hq_ctx *x, double *y, double rtol = 0.0) {
     const int N = x->N;
     const double *u = (const double *)x->Uh;
     const double na = 2.0 * N;
     if (rtol >= 1e-8 && x->ozgram && gram_oz_supported(2 * N) &&
         use_oz(x, 0.5 * (double)x->n * na * na)) {
-        // only the block <u, y> is used: the Gram's columns of y (the column
-        // tiles from y's first column on)
-        launch_gram_oz(x->n, u, N, y, N, x->h3, x->ozgram, x->Mw, x->status, x->st, N);
-        launch_extract(N, N, -1.0, x->Mw + N, 2 * N, x->Msm, N, x->st);
+        launch_gram_oz_xy(x->n, u, N, nullptr, 0, y, N, 2 * N, false, x->h3, x->ozgram, x->Ksm, x->status, x->st);
+        launch_extract(N, N, -1.0, x->Ksm, N, x->Msm, N, x->st);
     } else {
         GramPlan gp = make_gram_plan(x->n, N, N, false);
         launch_gram<double>(gp, u, N, nullptr, 0, y, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);

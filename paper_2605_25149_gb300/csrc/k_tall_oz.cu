@@ -5,24 +5,27 @@
 //
 // GB300 retires about two FP64 lane operations per clock per SM, so the FP64
 // SIMT form of these products is bound by the FP64 pipe.  Here every value is
-// written as a scaled sum of 8 signed 7-bit integer digits:
-//   A[p][k] = 2^(e_p) * sgn * sum_{i=1..8} a_i 2^(-7i)   (+ below 2^-56 |row max|),
+// written as a scaled sum of 7 balanced base-256 digits,
+//   A[p][k] = 2^(e_p + 1) sum_{i=1..7} a_i 2^(-8i)   (+- 2^-56 |row max|, rounded),
 // with e_p taken from the largest exponent of row p (points) of [A1 A2], and
-// likewise for each column c of [M1; M2].  Digits are integers 0..127, exact
-// in bf16.  Products of digit pairs with the same i + j = t share the scale
-// 2^(-7t) and are accumulated by kind::f16 MMAs into one FP32 TMEM
-// accumulator D_t; every partial sum is an integer below
-// 8 * K * 127^2 < 2^24 for K <= 128, so the accumulation is exact.  Pairs with
-// t <= 9 are kept (the dropped ones are below 2^-53 of |row max| |column max|
-// per term).  The epilogue combines D_2..D_9 in 64-bit fixed point, converts
+// likewise for each column c of [M1; M2].  Digits are integers -128..128, exact
+// in fp16.  Products of digit pairs with the same i + j = t share the scale
+// 2^(-8t) and are accumulated by kind::f16 MMAs into one FP32 TMEM
+// accumulator D_t; every partial sum is an integer of at most
+// 7 * K * 128^2 < 2^24 for K <= 128, so the accumulation is exact.  Pairs with
+// t <= 8 are kept (the dropped ones are below 2^-53 of |row max| |column max|
+// per term).  The epilogue combines D_2..D_8 in 64-bit fixed point, converts
 // once to FP64, applies 2^(e_p + f_c), adds Cin and optionally sums squares.
+// (Eight 7-bit sign-magnitude digits in bf16 have the same bounds but 36 digit
+// products instead of 28, and took 3.5 instead of 1.3 instructions per digit
+// to extract, where these kernels are bound by the integer pipe.)
 //
 // CTA = 128 points x 64 output columns, all K; per 64-wide K chunk the 512
 // threads (256 hid less of the latencies: 355 against 321 us at 64^3, K = 64)
-// convert the FP64 rows into 8 digit planes (K-major, 128-byte
-// swizzle) while bulk copies bring the 8 digit planes of the small matrix
-// (prepared once per call by k_oz_split); one thread issues the 36 digit
-// products of a K step of 16 as 12 MMAs.  TMEM: 8 accumulators x 64 columns = 512 columns.  The output
+// convert the FP64 rows into 7 digit planes (K-major, 128-byte
+// swizzle) while bulk copies bring the 7 digit planes of the small matrix
+// (prepared once per call by k_oz_split); one thread issues the 28 digit
+// products of a K step of 16 as 10 MMAs.  TMEM: 7 accumulators x 64 columns.  The output
 // tile is staged in the freed digit planes for whole-row Cin reads and Out
 // writes.  Every wait is bounded.
 #include "hq_internal.cuh"
@@ -36,9 +39,9 @@ namespace {
 
 constexpr int OZ_M = 128;                 // points per CTA (TMEM lanes)
 constexpr int OZ_NT = 64;                 // output columns per CTA
-constexpr int OZ_KC = 64;                 // K per chunk: 128 bytes of bf16 per row
-constexpr int OZ_S = 8;                   // digits per value
-constexpr int OZ_BITS = 7;                // bits per digit
+constexpr int OZ_KC = 64;                 // K per chunk: 128 bytes of fp16 per row
+constexpr int OZ_S = 7;                   // digits per value
+constexpr int OZ_BITS = 8;                // bits per digit
 constexpr int OZ_THREADS = 512;           // 16 warps: warp w reads TMEM lanes 32 (w % 4)..
 constexpr int OZ_EC = OZ_NT / (OZ_THREADS / 128);   // output columns per thread (16)
 constexpr int OZ_APLANE = OZ_M * 128;     // one digit plane of the point rows: 16 KB
@@ -56,13 +59,12 @@ __device__ __forceinline__ uint32_t sw128_offset16(int r, int k) {
                       ((k & 7) << 1));
 }
 
-// instruction descriptor: D f32, A/B bf16, both K-major
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-           ((uint32_t)(M >> 4) << 24);
+// instruction descriptor: D f32, A/B fp16, both K-major
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
                                          uint32_t accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
@@ -74,66 +76,74 @@ __device__ __forceinline__ int biased_exp(double x) {
     return (int)((__double_as_longlong(x) >> 52) & 0x7FF);
 }
 
-// |x| / 2^(emax - 1022) with 62 fraction bits (0 for zero, subnormal, Inf,
-// NaN), and the sign bit of x in bit 31
-__device__ __forceinline__ unsigned long long oz_fixed(double x, int emax, uint32_t &sgn) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7FF);
-    sgn = (uint32_t)(b >> 32) & 0x80000000u;
-    if (ex == 0 || ex == OZ_EBAD || emax == OZ_EBAD) return 0ull;
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const int sh = 9 + ex - emax;   // <= 9 since ex <= emax
-    return sh >= 0 ? (m << sh) : (sh > -64 ? (m >> (-sh)) : 0ull);
+// F + 0x4040404040404040 with F = x / 2^(emax - 1022) in 62-bit fixed point (0 for
+// zero and subnormals; unspecified for Inf and NaN, whose rows and columns the
+// exponent marks).  Digit i has its unit at bit 63 - 8i; the constant adds 128
+// units to each and half a unit of the last, so the digits are the bytes above
+// bit 6 less 128 (the first, of F up to 2^62, can reach 256 - 128).
+__device__ __forceinline__ unsigned long long oz_word(double x, int emax) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7FF), sg = (int)hi >> 31;
+    const uint32_t fh = (__funnelshift_l(lo, hi, 9) & 0x1FFFFFFFu) | 0x20000000u;
+    const int d = ex ? emax - ex : 64;   // >= 0; shifts of 64 and more give 0
+    unsigned long long f;
+    asm("shr.u64 %0, %1, %2;" : "=l"(f) : "l"(((unsigned long long)fh << 32) | (lo << 9)), "r"(d));
+    const long long s = sg;
+    return (f ^ (unsigned long long)s) + (0x4040404040404040ull - (unsigned long long)s);
 }
 
-// the 8 digits of two values of one row / column relative to the biased
-// exponent emax, as bf16 bit patterns of the signed integers, packed in
-// pairs plane by plane (x0 in the low half).  Digit i is bits
-// 55 - 7i .. 61 - 7i of the fixed-point magnitude; the signed integer +-d
-// comes from one float addition, (2^23 + d) - 2^23 with the sign of x on both
-// terms (+0 for d = 0), and its bf16 pattern is the upper half of the float.
+// the 7 digits of two values of one row / column relative to the biased
+// exponent emax as fp16 integers, packed in pairs plane by plane (x0 in the low
+// half): a byte b behind 0x64 is 1024 + b, less 1152
 __device__ __forceinline__ void oz_digits2(double x0, double x1, int emax, uint32_t (&pk)[OZ_S]) {
-    uint32_t s0, s1;
-    const unsigned long long f0 = oz_fixed(x0, emax, s0), f1 = oz_fixed(x1, emax, s1);
-    const uint32_t c0 = 0x4B000000u | s0, c1 = 0x4B000000u | s1;
-    const float a0 = s0 ? 8388608.0f : -8388608.0f, a1 = s1 ? 8388608.0f : -8388608.0f;
+    const unsigned long long w0 = oz_word(x0, emax), w1 = oz_word(x1, emax);
+    const uint32_t h0 = (uint32_t)(w0 >> 31), h1 = (uint32_t)(w1 >> 31);
+    const uint32_t l0 = (uint32_t)w0 << 1, l1 = (uint32_t)w1 << 1;
+    const uint32_t y23 = __byte_perm(h0, h1, 0x5612), y67 = __byte_perm(l0, l1, 0x5612);
+    pk[0] = __byte_perm((uint32_t)(w0 >> 55), (uint32_t)(w1 >> 55), 0x5410) | 0x64006400u;
+    pk[1] = __byte_perm(y23, 0x64u, 0x4240);
+    pk[2] = __byte_perm(y23, 0x64u, 0x4341);
+    pk[3] = (__byte_perm(h0, h1, 0x4400) & 0x00FF00FFu) | 0x64006400u;
+    pk[4] = (__byte_perm(l0, l1, 0x7733) & 0x00FF00FFu) | 0x64006400u;
+    pk[5] = __byte_perm(y67, 0x64u, 0x4240);
+    pk[6] = __byte_perm(y67, 0x64u, 0x4341);
 #pragma unroll
-    for (int i = 0; i < OZ_S; i++) {
-        const uint32_t d0 = (uint32_t)(f0 >> (62 - OZ_BITS * (i + 1))) & 127u;
-        const uint32_t d1 = (uint32_t)(f1 >> (62 - OZ_BITS * (i + 1))) & 127u;
-        const float v0 = __uint_as_float(c0 | d0) + a0;
-        const float v1 = __uint_as_float(c1 | d1) + a1;
-        pk[i] = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
-    }
+    for (int i = 0; i < OZ_S; i++) asm("sub.f16x2 %0, %0, %1;" : "+r"(pk[i]) : "r"(0x64806480u));
 }
 
-// sum_t D_t 2^(-7(t-2)), t = 2 .. 9, of 16 columns as 64-bit fixed point with FRAC
-// fraction bits.  Neighbouring digit sums join in 32 bits (128 D_t + D_{t+1}:
-// below 2^31 since |D_t| < 2^24 and only D_2 .. D_8 are shifted, |D_8| < 7 2^21),
-// the four halves in 64: q0 in units 2^-21, q1 in units 2^-49, of which one
-// truncation (below 2^-FRAC) remains.  tm: the thread's lane and first column.
+// sum_t D_t 2^(-8(t-2)), t = 2 .. 8, of 16 columns as 64-bit fixed point with FRAC
+// fraction bits (32 <= FRAC <= 48).  |D_t| <= (t - 1) 2^21: D_2 and D_3 join in 32
+// bits, the rest by wide multiply-adds; D_7 and D_8 are truncated once (below
+// 2^-FRAC).  tm: the thread's lane and first column.
 template <int FRAC>
 __device__ __forceinline__ void oz_combine(uint32_t tm, long long (&acc)[16], bool add) {
+    static_assert(OZ_S == 7 && OZ_BITS == 8 && FRAC >= 32 && FRAC <= 48, "");
 #pragma unroll
     for (int g = 0; g < 16; g += 8) {
-        long long q0[8];
-        int p[8];
+        const uint32_t c = tm + (uint32_t)g;
+        float a[8], b[8];
+        long long q[8];
+        int d[8];
+        tmem_ld8x2(c, c + OZ_NT, a, b);
 #pragma unroll
-        for (int h = 0; h < 4; h++) {
-            float a[8], b[8];
-            tmem_ld8x2(tm + (uint32_t)(2 * h * OZ_NT + g), tm + (uint32_t)((2 * h + 1) * OZ_NT + g), a, b);
+        for (int j = 0; j < 8; j++) d[j] = __float2int_rn(a[j]) * 256 + __float2int_rn(b[j]);
+        tmem_ld8x2(c + 2 * OZ_NT, c + 3 * OZ_NT, a, b);
 #pragma unroll
-            for (int j = 0; j < 8; j++) {
-                const int s = __float2int_rn(a[j]) * 128 + __float2int_rn(b[j]);
-                if ((h & 1) == 0) {
-                    p[j] = s;
-                } else {
-                    const long long q = (long long)p[j] * 16384 + s;
-                    if (h == 1) q0[j] = q << (FRAC - 21);
-                    else acc[g + j] = (add ? acc[g + j] : 0ll) + q0[j] + (q >> (49 - FRAC));
-                }
-            }
+        for (int j = 0; j < 8; j++) {
+            q[j] = ((long long)d[j] * 256 + __float2int_rn(a[j])) * 65536;   // units 2^-32
+            d[j] = __float2int_rn(b[j]);
         }
+        tmem_ld8x2(c + 4 * OZ_NT, c + 5 * OZ_NT, a, b);
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            q[j] += (long long)d[j] * 256 + __float2int_rn(a[j]);
+            d[j] = __float2int_rn(b[j]);
+        }
+        tmem_ld8(c + 6 * OZ_NT, a);
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+            acc[g + j] = (add ? acc[g + j] : 0ll) + (q[j] << (FRAC - 32)) +
+                         (((long long)d[j] * 256 + __float2int_rn(a[j])) >> (48 - FRAC));
     }
 }
 
@@ -145,7 +155,7 @@ __device__ __forceinline__ double pow2(int e) {
 }
 
 // Digit planes of the small matrix [M1; M2] (K x ncol) in the layout the MMA
-// reads: image[((ct * kchunks + ch) * 8 + j) * 8 KB] holds digit j of rows =
+// reads: image[((ct * kchunks + ch) * 7 + j) * 8 KB] holds digit j of rows =
 // output columns ct*64 .. +63 and K = ch*64 .. +63; fexp[c] = the column's
 // largest biased exponent.  CTA = one column tile; thread (kg, cl) takes
 // column cl and the pairs k = 2 (kg + SPL_G i), 2 (kg + SPL_G i) + 1 (the
@@ -206,6 +216,7 @@ __device__ __forceinline__ double oz_scaled(long long acc, int es) {
     if (u == 0) return 0.0;
     const int lz = __clzll((long long)u), ex = 1086 - lz + es;
     if (ex < 1 || ex > 2045) {   // subnormal or overflowing result
+        if (es < -1200) return 0.0;
         const double v = (double)acc;
         return es >= -1022 && es <= 1023 ? v * __longlong_as_double((long long)(es + 1023) << 52) : v * pow2(es);
     }
@@ -219,9 +230,10 @@ __device__ __forceinline__ double oz_scaled(long long acc, int es) {
 // allocation and its end cost a third of the one-tile-per-CTA form.  Per 64-wide
 // K chunk the digit planes are written in two halves of 32, and the MMAs of the
 // first run while the second is converted.  Measured at 64^3 points, K = 64, 64
-// columns: 334 -> 230 us (with Cin 375 -> 269); of a tile's 35,000 clocks the
-// conversion takes 6,000, the exposed MMAs 7,000, the epilogue 14,000 (removing
-// its arithmetic saves 6,000) and the output rows 3,200.
+// columns, with Cin: 375 -> 269 us, and 240 with the base-256 digits; of the
+// 35,000 clocks per tile before these the conversion took 6,000, the exposed MMAs
+// 7,000, the epilogue 14,000 (removing its arithmetic saved 6,000) and the output
+// rows 3,200.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_tall_oz(long n, int k1, int k2, int ncol, int kchunks, int ctiles, const double *__restrict__ A1,
               const double *__restrict__ A2, const unsigned char *__restrict__ image,
@@ -237,7 +249,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __shared__ __align__(16) int fexp_sh[OZ_NT];   // largest exponents of the tile's columns
     __shared__ int abort_sh, tmem_free_sh;
     __shared__ double red[OZ_THREADS / 32];
-    constexpr uint32_t TCOLS = OZ_S * OZ_NT;   // 512
+    constexpr uint32_t TCOLS = 512;   // OZ_S accumulators of 64, a power of two
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int K = k1 + k2;
@@ -352,23 +364,23 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                         for (int ks = 2 * h; ks < 2 * h + 2; ks++) {
-                            // digit i of A times digits j = 1 .. 9 - i of the small
+                            // digit i of A times digits j = 1 .. 8 - i of the small
                             // matrix: their planes follow each other as 64-row
                             // blocks of one B operand and so do the accumulators
-                            // D_{i+1} .. D_9, so up to four digits make one MMA of
-                            // 256 columns (12 MMAs in place of 36 of 64 columns,
+                            // D_{i+1} .. D_8, so up to four digits make one MMA of
+                            // 256 columns (10 MMAs in place of 28 of 64 columns,
                             // each of which took 80 clocks, the time A's rows take)
                             const uint32_t ko = ks * 32;
 #pragma unroll
                             for (int i = 1; i <= OZ_S; i++) {
                                 const uint64_t da = make_desc_sw128(smem_u32(planesA + (i - 1) * OZ_APLANE) + ko);
 #pragma unroll
-                                for (int j = 1; j <= 9 - i; j += 4) {
-                                    const int cnt = 10 - i - j < 4 ? 10 - i - j : 4;
+                                for (int j = 1; j <= OZ_S + 1 - i; j += 4) {
+                                    const int cnt = OZ_S + 2 - i - j < 4 ? OZ_S + 2 - i - j : 4;
                                     const uint64_t db =
                                         make_desc_sw128(smem_u32(planesB + (j - 1) * OZ_BPLANE) + ko);
-                                    mma_bf16(tmem + (uint32_t)((i + j - 2) * OZ_NT), da, db,
-                                             idesc_bf16(OZ_M, cnt * OZ_NT), (ch > 0 || ks > 0 || i > 1) ? 1u : 0u);
+                                    mma_f16(tmem + (uint32_t)((i + j - 2) * OZ_NT), da, db,
+                                             idesc_f16(OZ_M, cnt * OZ_NT), (ch > 0 || ks > 0 || i > 1) ? 1u : 0u);
                                 }
                             }
                         }
@@ -436,7 +448,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             double *sl = stg + r * OZ_SLD + cb;
 #pragma unroll
             for (int j = 0; j < OZ_EC; j++) {
-                const int es = (em - 1022) + (fc[j] - 1022) - 2 * OZ_BITS - OZ_FRAC;
+                const int es = (em - 1021) + (fc[j] - 1021) - 2 * OZ_BITS - OZ_FRAC;
                 double o = em == OZ_EBAD || fc[j] == OZ_EBAD ? __longlong_as_double(0x7FF8000000000000ll)
                                                              : oz_scaled(acc[j], es);
                 if (Cin) o += sl[j];
@@ -486,23 +498,32 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
-// FP64 Gram <X, X> = w X^T X of X = [X1 X2] (n x na, na <= 128) by the same
-// digit slicing, with per-column exponents over all points (k_oz_colexp).
-// CTA = all na rows x 64 output columns over a chunk of points; the digit
-// planes of a 32-point slice serve as both operands (the B operand is rows
-// ct*64.. of the A planes; 64-byte rows, 64-byte swizzle).  The planes of
-// OZ_GST slices are in flight: the converter warps fill slice s while the MMAs
-// of slice s-1 run.  The exact-sum bound holds for 128 points, so every four
-// slices the eight accumulators are read and added into 64-bit fixed-point
+// FP64 Grams by the same digit slicing, with per-column exponents over all
+// points (k_oz_colexp): <X, X> = w X^T X of X = [X1 X2] (n x na, na <= 128), or,
+// with a third block, <X, Y> = w X^T Y (Y: n x ny).
+// CTA = all na rows x 64 output columns over a chunk of points.  A slice of 32
+// points has the digit planes of the na rows (operand A) and, contiguously,
+// those of the tile's 64 columns (operand B: a second copy of the A rows
+// ct*64.., or Y's); 64-byte rows, 64-byte swizzle.  Contiguous planes make four
+// digits of B one MMA of up to 256 columns: 10 MMAs per 16 points (28 of 64
+// columns would take 80 clocks each).  Two slices are in flight: slice
+// s is converted while the MMAs of slice s - 1 run; 512 threads, of which one
+// issues the MMAs (a 17th warp for that cost every thread a fifth of its
+// registers: spills).  Bound by the integer instructions of the conversion and
+// the read-out: 64^3 points, 64 x 64 columns, X and Y separate: 219 -> 180 us
+// (36 products of 7-bit digits as MMAs of 64 columns; the same digits with this
+// schedule: 215).  The exact-sum bound holds for 128 points, so every four
+// slices the seven accumulators are read and added into 64-bit fixed-point
 // registers (OZ_GFRAC fraction bits); the chunk's FP64 partial tile is
 // summed over chunks in a fixed order by k_oz_gram_reduce.  D_t(i,j) and
-// D_t(j,i) are the same integers, so the result is exactly symmetric.
+// D_t(j,i) are the same integers, so <X, X> is exactly symmetric.
 // ---------------------------------------------------------------------------
 constexpr int OZ_GFRAC = 32;
 constexpr int OZ_GKC = 32;                       // points per slice: 64-byte rows
-constexpr int OZ_GPLANE = OZ_M * 64;             // one digit plane of a slice: 8 KB
-constexpr int OZ_GSTAGE = OZ_S * OZ_GPLANE;      // the eight planes: 64 KB
-constexpr int OZ_GST = 3;                        // slices in flight
+constexpr int OZ_GPLANE = OZ_M * 64;             // one digit plane of a slice's rows: 8 KB
+constexpr int OZ_GBPLANE = OZ_NT * 64;           // and of its columns: 4 KB
+constexpr int OZ_GSTAGE = OZ_S * (OZ_GPLANE + OZ_GBPLANE);   // the planes of a slice: 84 KB
+constexpr int OZ_GST = 2;                        // slices in flight
 constexpr int OZ_GFLUSH = 128 / OZ_GKC;          // slices per exact accumulation
 constexpr int OZ_GSMEM = OZ_GST * OZ_GSTAGE + 2048;   // + alignment slack
 
@@ -524,52 +545,67 @@ __device__ __forceinline__ uint64_t make_desc_sw64(uint32_t saddr) {
     return d;
 }
 
-__global__ void __launch_bounds__(128) k_oz_colexp(long n, int n1, int n2, const double *X1,
+// colexp[c] = the largest biased exponent of column c of [X1 X2] (zeroed before)
+__global__ void __launch_bounds__(256) k_oz_colexp(long n, int n1, int n2, const double *X1,
                                                    const double *X2, int *colexp) {
-    const int c = threadIdx.x, na = n1 + n2;
-    if (c >= na) return;
+    const int na = n1 + n2, per = 256 / na;   // rows per pass of the CTA
+    const int c = threadIdx.x % na, g = threadIdx.x / na;
+    if (g >= per) return;
+    const double *src = c < n1 ? X1 + c : X2 + (c - n1);
+    const size_t ld = c < n1 ? n1 : n2;
+    const long step = (long)gridDim.x * per;
     int em = 0;
-    for (long p = blockIdx.x; p < n; p += gridDim.x)
-        em = max(em, biased_exp(c < n1 ? X1[(size_t)p * n1 + c] : X2[(size_t)p * n2 + (c - n1)]));
+    for (long p = (long)blockIdx.x * per + g; p < n; p += 4 * step) {
+        int e[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) e[u] = p + u * step < n ? biased_exp(src[(size_t)(p + u * step) * ld]) : 0;
+        em = max(em, max(max(e[0], e[1]), max(e[2], e[3])));
+    }
     atomicMax(&colexp[c], em);
 }
 
-// 16 converter warps (digit planes, TMEM read-out, epilogue) and one warp
-// whose first lane issues the MMAs; they meet only at mbarriers: full[st]
-// (the planes of a slice are written), done[st] (its MMAs completed, the
-// stage is free) and tfree (the accumulators were read out at a flush)
-constexpr int OZ_GCONV = 512;
-constexpr int OZ_GTHREADS = OZ_GCONV + 32;
+// 512 threads convert; they meet at mbarriers: full[st] (the planes of a slice
+// are written; OZ_GISSUE issues its MMAs), done[st] (these completed, the stage is
+// free) and tfree (the accumulators were read out at a flush)
+constexpr int OZ_GTHREADS = 512;
+constexpr int OZ_GISSUE = OZ_GTHREADS - 32;   // of the warp with the fewest units
 
+template <bool HASY>
 __global__ void __launch_bounds__(OZ_GTHREADS, 1)
-    k_gram_oz(long n, int n1, int n2, long chunk_rows, int ct0, const double *__restrict__ X1,
-              const double *__restrict__ X2, const int *__restrict__ colexp,
-              double *__restrict__ partials, int *status) {
+    k_gram_oz(long n, int n1, int n2, int ny, long chunk_rows, const double *__restrict__ X1,
+              const double *__restrict__ X2, const double *__restrict__ Y, const int *__restrict__ colexp,
+              const int *__restrict__ yexp, double *__restrict__ partials, int *status) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *planes = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t full[OZ_GST], done[OZ_GST], tfree;
     __shared__ uint32_t tmem_base_sh;
-    __shared__ int cexp[OZ_M];
+    __shared__ int cexp[OZ_M], bexp[OZ_NT];   // exponents of the rows, of the tile's columns
     __shared__ volatile int abort_sh;
     __shared__ int last_sh, tmem_free_sh;
-    constexpr uint32_t TCOLS = OZ_S * OZ_NT;   // 512
+    constexpr uint32_t TCOLS = 512;   // OZ_S accumulators of 64, a power of two
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int na = n1 + n2, ct = ct0 + blockIdx.x;   // output column tile
+    const int na = n1 + n2, ct = blockIdx.x;   // output column tile
+    const int nb = HASY ? ny : na;                   // output columns
     const long p0 = (long)blockIdx.y * chunk_rows;
     const long p1 = (n < p0 + chunk_rows) ? n : p0 + chunk_rows;
     const int nslices = p1 > p0 ? (int)((p1 - p0 + OZ_GKC - 1) / OZ_GKC) : 0;
     if (tid == 0) {
         for (int i = 0; i < OZ_GST; i++) {
-            mbar_init(&full[i], OZ_GCONV);
+            mbar_init(&full[i], OZ_GTHREADS);
             mbar_init(&done[i], 1);
         }
-        mbar_init(&tfree, OZ_GCONV);
+        mbar_init(&tfree, OZ_GTHREADS);
         abort_sh = 0;
         last_sh = -1;   // last slice whose MMAs were committed
         tmem_free_sh = 1;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int c = tid; c < OZ_M; c += OZ_GTHREADS) cexp[c] = c < na ? colexp[c] : 0;
+    if (tid < OZ_M) cexp[tid] = tid < na ? colexp[tid] : 0;
+    if (tid < OZ_NT) bexp[tid] = ct * OZ_NT + tid < nb ? (HASY ? yexp : colexp)[ct * OZ_NT + tid] : 0;
+    // rows and columns beyond the blocks keep these zero digits
+    if (na < OZ_M || nb < (ct + 1) * OZ_NT)
+        for (int t = tid; t < OZ_GST * OZ_GSTAGE / 16; t += OZ_GTHREADS)
+            reinterpret_cast<uint4 *>(planes)[t] = make_uint4(0, 0, 0, 0);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_base_sh)),
@@ -582,14 +618,14 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base_sh;
     // completion of the MMAs of slice q: the (q / OZ_GST)-th commit on
-    // done[q % OZ_GST].  No role can run a phase ahead of the one another
-    // role waits for (each next arrival needs the awaited phase), so every
+    // done[q % OZ_GST].  No thread can run a phase ahead of the one another
+    // waits for (each next arrival needs the awaited phase), so every
     // parity below is unambiguous.
     auto wait_done = [&](int q) -> bool {
         return mbar_wait(&done[q % OZ_GST], (unsigned)((q / OZ_GST) & 1));
     };
-    // fixed-point sums: converter thread = TMEM lane 32 (warp % 4) + lane
-    // (Gram row), 16 output columns (warp / 4)
+    // fixed-point sums: thread = TMEM lane 32 (warp % 4) + lane (Gram row), 16
+    // output columns (warp / 4)
     const int grow = (warp & 3) * 32 + lane, gcb = (warp >> 2) * 16;
     long long facc[16];
 #pragma unroll
@@ -597,129 +633,139 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
     auto flush = [&]() {
         oz_combine<OZ_GFRAC>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)gcb, facc, true);
     };
-    if (warp == OZ_GCONV / 32) {
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16(OZ_M, OZ_NT);
-            for (int sl = 0; sl < nslices; sl++) {
-                if (abort_sh) break;
-                const int st = sl % OZ_GST;
-                const bool fresh = sl % OZ_GFLUSH == 0;
-                if (!mbar_wait(&full[st], (unsigned)((sl / OZ_GST) & 1)) ||
-                    (fresh && sl > 0 && !mbar_wait(&tfree, (unsigned)((sl / OZ_GFLUSH - 1) & 1)))) {
-                    abort_sh = 1;
-                    break;
+    // the MMAs of slice sl (one thread): digit i of the rows times up to four
+    // digits j of the columns, j <= 8 - i, into D_{i + j}..; i = 1 reaches all
+    // seven accumulators, so it comes first and starts a fresh sum
+    auto issue = [&](int sl, bool fresh) {
+        const uint32_t stage = smem_u32(planes + (sl % OZ_GST) * OZ_GSTAGE);
+#pragma unroll
+        for (int ks = 0; ks < OZ_GKC / 16; ks++) {
+            const uint32_t ko = ks * 32;
+#pragma unroll
+            for (int i = 1; i <= OZ_S; i++) {
+                const uint64_t da = make_desc_sw64(stage + (i - 1) * OZ_GPLANE + ko);
+#pragma unroll
+                for (int j = 1; j <= OZ_S + 1 - i; j += 4) {
+                    const int nd = OZ_S + 2 - i - j < 4 ? OZ_S + 2 - i - j : 4;
+                    const uint64_t db = make_desc_sw64(stage + OZ_S * OZ_GPLANE + (j - 1) * OZ_GBPLANE + ko);
+                    mma_f16(tmem + (uint32_t)((i + j - 2) * OZ_NT), da, db, idesc_f16(OZ_M, nd * OZ_NT),
+                             fresh && ks == 0 && i == 1 ? 0u : 1u);
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                unsigned char *stage = planes + st * OZ_GSTAGE;
-#pragma unroll
-                for (int ks = 0; ks < OZ_GKC / 16; ks++) {
-                    const uint32_t ko = ks * 32;
-#pragma unroll
-                    for (int t = 2; t <= OZ_S + 1; t++) {
-                        const int ilo = t - OZ_S > 1 ? t - OZ_S : 1;
-                        const int ihi = t - 1 < OZ_S ? t - 1 : OZ_S;
-#pragma unroll
-                        for (int i = ilo; i <= ihi; i++) {
-                            const int j = t - i;
-                            const uint64_t da =
-                                make_desc_sw64(smem_u32(stage + (i - 1) * OZ_GPLANE) + ko);
-                            const uint64_t db = make_desc_sw64(
-                                smem_u32(stage + (j - 1) * OZ_GPLANE + ct * OZ_NT * 64) + ko);
-                            const uint32_t acc = (!fresh || ks > 0 || i > ilo) ? 1u : 0u;
-                            mma_bf16(tmem + (uint32_t)((t - 2) * OZ_NT), da, db, idesc, acc);
-                        }
-                    }
-                }
-                mma_commit(&done[st]);
-                last_sh = sl;
             }
         }
-    } else {
-        // slice loads: thread t takes column c = t & 127 of the 8 consecutive
-        // points 8 (t >> 7) + j (coalesced across the lanes for each j)
-        const int lc = tid & (OZ_M - 1), lq = tid >> 7;
-        double xv[8];
-        auto load_slice = [&](int sl) {
+        mma_commit(&done[sl % OZ_GST]);
+        last_sh = sl;
+    };
+    // Conversion units: 16 columns (of X, then of Y, each padded to 16) x 8 points
+    // per warp; lane = column lane >> 1, points 4 (lane & 1) .. + 3, so that the
+    // lanes of a column fill one 16-byte chunk of each digit plane (no bank
+    // conflicts) and loads are 128-byte rows.  A unit's values of the next slice
+    // are loaded as soon as it is converted, under the conversion of the others.
+    constexpr int U = HASY ? 3 : 2;
+    const int ga = (na + 15) / 16, ng = ga + (HASY ? (min(ny - ct * OZ_NT, OZ_NT) + 15) / 16 : 0);
+    const double *src[U];   // the unit's first point of slice 0 (null: none)
+    int ld[U], ue[U], pt[U];
+    uint32_t off[U], offb[U];   // first plane of the values, and of their copy (offb != 0)
 #pragma unroll
-            for (int j = 0; j < 8; j++) {
-                const long p = p0 + (long)sl * OZ_GKC + 8 * lq + j;
-                xv[j] = (p < p1 && lc < na)
-                            ? (lc < n1 ? X1[(size_t)p * n1 + lc] : X2[(size_t)p * n2 + (lc - n1)])
-                            : 0.0;
-            }
-        };
-        const int em = cexp[lc];
-        if (nslices > 0) load_slice(0);
-        for (int sl = 0; sl < nslices; sl++) {
-            if (abort_sh) break;
-            const int st = sl % OZ_GST;
-            const bool fresh = sl % OZ_GFLUSH == 0;
-            // the stage's previous slice is consumed
-            if (sl >= OZ_GST && !wait_done(sl - OZ_GST)) {
+    for (int k = 0; k < U; k++) {
+        const int wu = warp + k * (OZ_GTHREADS / 32), grp = wu % ng, oct = wu / ng;
+        const bool isy = HASY && grp >= ga;
+        const int c = (isy ? grp - ga : grp) * 16 + (lane >> 1);   // row of the planes
+        const int col = isy ? ct * OZ_NT + c : c;
+        src[k] = nullptr;
+        ld[k] = ue[k] = 0;
+        off[k] = offb[k] = 0;
+        pt[k] = 8 * oct + 4 * (lane & 1);
+        if (oct >= OZ_GKC / 8 || col >= (isy ? ny : na)) continue;
+        ld[k] = isy ? ny : (col < n1 ? n1 : n2);
+        src[k] = (isy ? Y + col : (col < n1 ? X1 + col : X2 + (col - n1))) + (size_t)(p0 + pt[k]) * ld[k];
+        ue[k] = isy ? bexp[c] : cexp[c];
+        off[k] = (isy ? OZ_S * OZ_GPLANE : 0) + sw64_offset16(c, pt[k]);
+        const int bc = c - ct * OZ_NT;
+        if (!HASY && bc >= 0 && bc < OZ_NT) offb[k] = OZ_S * OZ_GPLANE + sw64_offset16(bc, pt[k]);
+    }
+    double xv[U][4];
+    auto load = [&](int sl, int k) {
+        const long left = src[k] ? p1 - p0 - (long)sl * OZ_GKC - pt[k] : 0;   // points there are
+        const double *q = src[k] + (size_t)sl * OZ_GKC * ld[k];
+#pragma unroll
+        for (int j = 0; j < 4; j++) xv[k][j] = j < left ? q[(size_t)j * ld[k]] : 0.0;
+    };
+    if (nslices > 0)
+#pragma unroll
+        for (int k = 0; k < U; k++) load(0, k);
+    for (int sl = 0; sl < nslices; sl++) {
+        if (abort_sh) break;
+        const int st = sl % OZ_GST;
+        const bool fresh = sl % OZ_GFLUSH == 0;
+        // the stage's previous slice is consumed
+        if (sl >= OZ_GST && !wait_done(sl - OZ_GST)) {
+            abort_sh = 1;
+            break;
+        }
+        unsigned char *stage = planes + st * OZ_GSTAGE;
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+            if (!src[k]) continue;
+            uint32_t lo[OZ_S], hi[OZ_S];
+            oz_digits2(xv[k][0], xv[k][1], ue[k], lo);
+            oz_digits2(xv[k][2], xv[k][3], ue[k], hi);
+            if (sl + 1 < nslices) load(sl + 1, k);
+            const uint32_t ps = HASY && off[k] >= OZ_S * OZ_GPLANE ? OZ_GBPLANE : OZ_GPLANE;
+#pragma unroll
+            for (int i = 0; i < OZ_S; i++)
+                *reinterpret_cast<uint2 *>(stage + off[k] + i * ps) = make_uint2(lo[i], hi[i]);
+            if (!HASY && offb[k])
+#pragma unroll
+                for (int i = 0; i < OZ_S; i++)
+                    *reinterpret_cast<uint2 *>(stage + offb[k] + i * OZ_GBPLANE) = make_uint2(lo[i], hi[i]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(&full[st]);
+        if (fresh && sl > 0) {
+            // 128 points accumulated: every MMA so far is complete
+            if (!wait_done(sl - 1)) {
                 abort_sh = 1;
                 break;
             }
-            if (fresh && sl > 0) {
-                // 128 points accumulated: every MMA so far is complete
-                if (!wait_done(sl - 1)) {
-                    abort_sh = 1;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                flush();
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive(&tfree);
-            }
-            // eight consecutive points of one column: one 16-byte chunk of
-            // each digit plane
-            {
-                uint32_t pk[OZ_S][4];
-#pragma unroll
-                for (int u = 0; u < 8; u += 2) {
-                    uint32_t pp[OZ_S];
-                    oz_digits2(xv[u], xv[u + 1], em, pp);
-#pragma unroll
-                    for (int i = 0; i < OZ_S; i++) pk[i][u >> 1] = pp[i];
-                }
-                unsigned char *stage = planes + st * OZ_GSTAGE;
-                const uint32_t off = sw64_offset16(lc, 8 * lq);
-#pragma unroll
-                for (int i = 0; i < OZ_S; i++)
-                    *reinterpret_cast<uint4 *>(stage + i * OZ_GPLANE + off) =
-                        make_uint4(pk[i][0], pk[i][1], pk[i][2], pk[i][3]);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive(&full[st]);
-            if (sl + 1 < nslices) load_slice(sl + 1);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            flush();
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(&tfree);
         }
-        if (!abort_sh && nslices > 0 && !wait_done(nslices - 1)) abort_sh = 1;
+        if (tid == OZ_GISSUE) {
+            if (!mbar_wait(&full[st], (unsigned)((sl / OZ_GST) & 1)) ||
+                (fresh && sl > 0 && !mbar_wait(&tfree, (unsigned)((sl / OZ_GFLUSH - 1) & 1)))) {
+                abort_sh = 1;
+            } else {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                issue(sl, fresh);
+            }
+        }
     }
+    if (!abort_sh && nslices > 0 && !wait_done(nslices - 1)) abort_sh = 1;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // after a wait that gave up, one more bounded wait for the last commit
     // before the columns are released (if it fails too they stay allocated,
     // and only the status word is meaningful)
-    if (tid == OZ_GCONV && abort_sh && last_sh >= 0) tmem_free_sh = wait_done(last_sh) ? 1 : 0;
+    if (tid == OZ_GISSUE && abort_sh && last_sh >= 0) tmem_free_sh = wait_done(last_sh) ? 1 : 0;
     __syncthreads();
     if (abort_sh) {
         if (tid == 0) atomicOr(status, ST_TC_TIMEOUT);
-    } else if (tid < OZ_GCONV) {
+    } else {
         if (nslices > 0) flush();
         double *dst = partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * OZ_M * OZ_NT;
         const int ea = cexp[grow];
 #pragma unroll
         for (int j = 0; j < 16; j++) {
-            const int gc = ct * OZ_NT + gcb + j;
             double o = 0.0;
-            if (grow < na && gc < na) {
-                const int eb = cexp[gc];
-                const int es = (ea - 1022) + (eb - 1022) - 2 * OZ_BITS - OZ_GFRAC;
-                if (ea == OZ_EBAD || eb == OZ_EBAD) o = __longlong_as_double(0x7FF8000000000000ll);
-                else if (es >= -1022 && es <= 1023)
-                    o = (double)facc[j] * __longlong_as_double((long long)(es + 1023) << 52);
-                else
-                    o = (double)facc[j] * pow2(es);
+            if (grow < na && ct * OZ_NT + gcb + j < nb) {
+                const int eb = bexp[gcb + j];
+                const int es = (ea - 1021) + (eb - 1021) - 2 * OZ_BITS - OZ_GFRAC;
+                o = ea == OZ_EBAD || eb == OZ_EBAD ? __longlong_as_double(0x7FF8000000000000ll)
+                                                   : oz_scaled(facc[j], es);
             }
             dst[(size_t)grow * OZ_NT + gcb + j] = o;
         }
@@ -731,17 +777,16 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
                      : "memory");
 }
 
-// out[i][j] = w * sum over chunks of the chunk partials, for the columns of the
-// ctiles tiles from tile ct0 on (the others are not written).  CTA = 32
-// entries x 8 threads, each summing an eighth of the chunks in order, then the
-// eighths in order (one thread per entry waited for 152 dependent loads: 42 us
-// at na = 128; see k_gram_reduce)
-__global__ void __launch_bounds__(256) k_oz_gram_reduce(int na, int ct0, int ctiles, int chunks,
+// out[i][j] = w * sum over chunks of the chunk partials (na x nb, row-major).
+// CTA = 32 entries x 8 threads, each summing an eighth of the chunks in order,
+// then the eighths in order (one thread per entry waited for 152 dependent
+// loads: 42 us at na = 128; see k_gram_reduce)
+__global__ void __launch_bounds__(256) k_oz_gram_reduce(int na, int nb, int ctiles, int chunks,
                                                         const double *partials, double w, double *out) {
     __shared__ double red[8][33];
     const int e = blockIdx.x * 32 + threadIdx.x, g = threadIdx.y;
-    const int i = e / na, j = e % na, ct = j / OZ_NT - ct0, jl = j % OZ_NT;
-    const bool ok = e < na * na && ct >= 0;
+    const int i = e / nb, j = e % nb, ct = j / OZ_NT, jl = j % OZ_NT;
+    const bool ok = e < na * nb;
     const int per = (chunks + 7) / 8, c0 = min(chunks, g * per), c1 = min(chunks, c0 + per);
     const size_t stride = (size_t)ctiles * OZ_M * OZ_NT;
     red[g][threadIdx.x] =
@@ -772,7 +817,8 @@ void oz_prepare() {
     static bool done = false;
     if (done) return;
     cudaFuncSetAttribute(k_tall_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
-    cudaFuncSetAttribute(k_gram_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_GSMEM);
+    cudaFuncSetAttribute(k_gram_oz<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_GSMEM);
+    cudaFuncSetAttribute(k_gram_oz<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_GSMEM);
     done = true;
 }
 
@@ -783,12 +829,13 @@ struct OzGramPlan {
     int ctiles, chunks;
     long chunk_rows;
 };
-OzGramPlan make_oz_gram_plan(long n, int na) {
+// nb output columns
+OzGramPlan make_oz_gram_plan(long n, int nb) {
     OzGramPlan g;
-    g.ctiles = (na + OZ_NT - 1) / OZ_NT;
-    // at most 16384 points per chunk: the 64-bit fixed-point sums then stay
-    // below 2^60 (2^53 per 128-point flush)
-    long chunks = std::max((long)(2 * 152) / g.ctiles, (n + 16383) / 16384);
+    g.ctiles = (nb + OZ_NT - 1) / OZ_NT;
+    // one CTA per SM; at most 16384 points per chunk: the 64-bit fixed-point
+    // sums then stay below 2^60 (2^53 per 128-point flush)
+    long chunks = std::max((long)152 / g.ctiles, (n + 16383) / 16384);
     chunks = std::max(1L, std::min(chunks, (n + OZ_KC - 1) / OZ_KC));
     long rows = (n + chunks - 1) / chunks;
     rows = (rows + OZ_KC - 1) / OZ_KC * OZ_KC;
@@ -796,29 +843,52 @@ OzGramPlan make_oz_gram_plan(long n, int na) {
     g.chunks = (int)((n + rows - 1) / rows);
     return g;
 }
+size_t oz_gram_tiles(long n, int nb) {
+    const OzGramPlan g = make_oz_gram_plan(n, nb);
+    return (size_t)g.chunks * g.ctiles;
+}
+int *oz_exponents(double *scratch, long n, int na) {
+    return reinterpret_cast<int *>(scratch + std::max(oz_gram_tiles(n, na), oz_gram_tiles(n, OZ_NT)) * OZ_M * OZ_NT);
+}
+void oz_colexp(long n, const double *X1, int n1, const double *X2, int n2, int *colexp, cudaStream_t s) {
+    cudaMemsetAsync(colexp, 0, sizeof(int) * OZ_M, s);
+    HQ_LAUNCH(HQ_K_GRAM, k_oz_colexp<<<1024, 256, 0, s>>>(n, n1, n2, X1, X2, colexp));
+}
 }  // namespace
 
+// the exponents of the rows and of a separate block's columns follow the partials
+// of na or OZ_NT output columns, whichever are more
 size_t gram_oz_scratch_bytes(long n, int na) {
-    OzGramPlan g = make_oz_gram_plan(n, na);
-    return sizeof(double) * (size_t)g.chunks * g.ctiles * OZ_M * OZ_NT + sizeof(int) * OZ_M;
+    return sizeof(double) * std::max(oz_gram_tiles(n, na), oz_gram_tiles(n, OZ_NT)) * OZ_M * OZ_NT +
+           sizeof(int) * 2 * OZ_M;
 }
 
 void launch_gram_oz(long n, const double *X1, int n1, const double *X2, int n2, double w,
-                    double *scratch, double *out, int *status, cudaStream_t s, int col0) {
+                    double *scratch, double *out, int *status, cudaStream_t s) {
     if (!X2) n2 = 0;
     const int na = n1 + n2;
-    OzGramPlan g = make_oz_gram_plan(n, na);
-    // output columns from the tile holding column col0 on
-    const int ct0 = std::min(std::max(col0, 0) / OZ_NT, g.ctiles - 1), nt = g.ctiles - ct0;
-    double *partials = scratch;
-    int *colexp = reinterpret_cast<int *>(scratch + (size_t)g.chunks * g.ctiles * OZ_M * OZ_NT);
-    cudaMemsetAsync(colexp, 0, sizeof(int) * OZ_M, s);
-    HQ_LAUNCH(HQ_K_GRAM, k_oz_colexp<<<1024, 128, 0, s>>>(n, n1, n2, X1, n2 ? X2 : nullptr, colexp));
-    HQ_LAUNCH(HQ_K_GRAM, k_gram_oz<<<dim3(nt, g.chunks), OZ_GTHREADS, OZ_GSMEM, s>>>(
-                             n, n1, n2, g.chunk_rows, ct0, X1, n2 ? X2 : nullptr, colexp, partials,
-                             status));
-    HQ_LAUNCH(HQ_K_GRAM, k_oz_gram_reduce<<<(na * na + 31) / 32, dim3(32, 8), 0, s>>>(
-                             na, ct0, nt, g.chunks, partials, w, out));
+    const OzGramPlan g = make_oz_gram_plan(n, na);
+    int *colexp = oz_exponents(scratch, n, na);
+    oz_colexp(n, X1, n1, X2, n2, colexp, s);
+    HQ_LAUNCH(HQ_K_GRAM, k_gram_oz<false><<<dim3(g.ctiles, g.chunks), OZ_GTHREADS, OZ_GSMEM, s>>>(
+                             n, n1, n2, 0, g.chunk_rows, X1, X2, nullptr, colexp, nullptr, scratch, status));
+    HQ_LAUNCH(HQ_K_GRAM, k_oz_gram_reduce<<<(na * na + 31) / 32, dim3(32, 8), 0, s>>>(na, na, g.ctiles, g.chunks,
+                                                                                      scratch, w, out));
+}
+
+void launch_gram_oz_xy(long n, const double *X1, int n1, const double *X2, int n2, const double *Y, int ny,
+                       int na_scratch, bool have_xexp, double w, double *scratch, double *out, int *status,
+                       cudaStream_t s) {
+    if (!X2) n2 = 0;
+    const int na = n1 + n2;
+    const OzGramPlan g = make_oz_gram_plan(n, ny);
+    int *xexp = oz_exponents(scratch, n, na_scratch), *yexp = xexp + OZ_M;
+    if (!have_xexp) oz_colexp(n, X1, n1, X2, n2, xexp, s);
+    oz_colexp(n, Y, ny, nullptr, 0, yexp, s);
+    HQ_LAUNCH(HQ_K_GRAM, k_gram_oz<true><<<dim3(g.ctiles, g.chunks), OZ_GTHREADS, OZ_GSMEM, s>>>(
+                             n, n1, n2, ny, g.chunk_rows, X1, X2, Y, xexp, yexp, scratch, status));
+    HQ_LAUNCH(HQ_K_GRAM, k_oz_gram_reduce<<<(na * ny + 31) / 32, dim3(32, 8), 0, s>>>(na, ny, g.ctiles, g.chunks,
+                                                                                      scratch, w, out));
 }
 
 void launch_tall_oz(long n, const double *A1, int k1, const double *M1, const double *A2, int k2,
