@@ -304,6 +304,10 @@ void launch_rowreduce(int mode, long n, int N, const double *u, const double *v,
 void launch_scale_rows(long n, int N, const double *g, const double *u, double *y, cudaStream_t s);
 void launch_shift_cols(long n, int N, const double *sft, const double *x, double *y,
                        cudaStream_t s);
+void launch_apply_shifted(const GridGeom &g, const double *D, double c, const double *x, const double *shifts,
+                          double *y, double *part_xy, cudaStream_t s);
+void launch_newton_project(int N, bool first, const double *K, const double *beta, double *Cneg, double *G,
+                           cudaStream_t s);
 // An FP32 preconditioner inside an FP64 block PCG, its interface fused into
 // the PCG passes (g: the FP64 geometry of the finest level for the PCG
 // kernels, the FP32 one for the sweep):

@@ -139,7 +139,8 @@ __device__ __forceinline__ VT<T, V> nbr_sum(const T *__restrict__ x, size_t e, i
 }
 
 // ---------------------------------------------------------------------------
-// 7-point operator.  MODE 0: y = A x (+ x.y);  MODE 1: y = b - A x (+ y.y, b.b)
+// 7-point operator.  MODE 0: y = A x (+ x.y);  MODE 1: y = b - A x (+ y.y, b.b);
+// MODE 2: y = A x - b o x with b one shift per column (+ x.y)
 // A x = D x - c (x_w + x_e + x_s + x_n + x_b + x_t),  D = 6c + V + sigma.
 // The residual is formed as (b - D x) + c s: two FMAs after the neighbour
 // sum, one FP64-pipe instruction fewer than b - (D x - c s).
@@ -177,6 +178,9 @@ __global__ void __launch_bounds__(256) k_stencil(int m, long n, int N, int ppt,
 #pragma unroll
         for (int v = 0; v < V; v++)
             o.v[v] = MODE == 1 ? resid_value(bb.v[v], d, xc.v[v], c, s.v[v]) : op_value(d, xc.v[v], c, s.v[v]);
+        if (MODE == 2)
+#pragma unroll
+            for (int v = 0; v < V; v++) o.v[v] -= b[col + v] * xc.v[v];
         if (MODE == 1) {
 #pragma unroll
             for (int v = 0; v < V; v++) {
@@ -423,6 +427,7 @@ __global__ void __launch_bounds__(256) k_stencil_zm(int m, int N, int nseg, int 
                 const T sum = sum6(a, in);
                 o.v[v] = MODE == 1 ? resid_value(bb.v[v], d, xcur.v[v], c, sum)
                                    : op_value(d, xcur.v[v], c, sum);
+                if (MODE == 2) o.v[v] -= b[col + v] * xcur.v[v];
             }
             if (MODE == 1) {
 #pragma unroll
@@ -905,6 +910,18 @@ void launch_shift_cols(long n, int N, const double *sft, const double *x, double
 }
 
 //   out[e] = a * x[e] + b * y[e]            (whole blocks, FP64)
+// of a Newton solve's Gram K = [C; E] (2N x N): Cneg = -C, G = E + beta_j G (column
+// j; first: G = E)
+__global__ void k_newton_project(int N, int first, const double *K, const double *beta, double *Cneg, double *G) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < N * N; t += gridDim.x * blockDim.x) {
+        Cneg[t] = -K[t];
+        G[t] = first ? K[N * N + t] : fma(beta[t % N], G[t], K[N * N + t]);
+    }
+}
+void launch_newton_project(int N, bool first, const double *K, const double *beta, double *Cneg, double *G,
+                           cudaStream_t s) {
+    HQ_LAUNCH(HQ_K_SMALL, k_newton_project<<<(N * N + 255) / 256, 256, 0, s>>>(N, first, K, beta, Cneg, G));
+}
 __global__ void k_axpby(size_t count, double a, const double *x, double b, const double *y,
                         double *out) {
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count;
@@ -1301,6 +1318,25 @@ template <typename T>
 void launch_apply(const GridGeom &g, const T *D, T c, const T *x, T *y, double *part_xy,
                   cudaStream_t s) {
     HQ_VEC_DISPATCH(T, g, run_apply, g, D, c, x, y, part_xy, s);
+}
+
+// y = (A - diag(shifts)) x, the shift per column, and the partials of x.y: one pass
+// of the projected PCG instead of the operator, a shift pass (60 us at 64^3, 64
+// columns) and a dot product (43 us)
+template <typename T, int V>
+static void run_apply_shifted(const GridGeom &g, const T *D, T c, const T *x, const T *sh, T *y, double *part,
+                              cudaStream_t s) {
+    const double el = (double)g.n * g.N;
+    if (g.zch > 0)
+        HQ_LAUNCH_W(HQ_K_STENCIL, el, k_stencil_zm<T, V, 2, true><<<zm_grid(g), blk(g), 0, s>>>(
+                                          g.m, g.N, zm_segments(g), zm_planes(g), D, c, x, sh, y, part, nullptr));
+    else
+        HQ_LAUNCH_W(HQ_K_STENCIL, el, k_stencil<T, V, 2, true><<<grd(g), blk(g), 0, s>>>(
+                                          g.m, g.n, g.N, g.ppt, D, c, x, sh, y, part, nullptr));
+}
+void launch_apply_shifted(const GridGeom &g, const double *D, double c, const double *x, const double *shifts,
+                          double *y, double *part_xy, cudaStream_t s) {
+    HQ_VEC_DISPATCH(double, g, run_apply_shifted, g, D, c, x, shifts, y, part_xy, s);
 }
 
 template <typename T, int V>
