@@ -352,11 +352,20 @@ void launch_gram_tc(long n, const float *X1, int n1, const float *X2, int n2, do
 // full (worker warps arrive), B stage full (bulk-copy bytes), stage empty
 // and accumulator full (MMA commits), accumulator empty (worker warps), so
 // the MMAs of one slice overlap the split of the next ones and the write-out
-// of a finished work item.
+// of a finished work item.  A slice is read out two slices later, from one of four
+// accumulators (read out one later, every slice waited for its predecessor's
+// MMAs), A slices are loaded two ahead.  Measured at 64^3 points, K = 256, 128
+// columns: 208 -> 169 us.  Bound by the workers' instruction latency with nine
+// warps on the SM: without the A loads' DRAM traffic, the B copies, the read-out
+// or 11 of 12 MMAs it still takes 155 - 171; sixteen workers (a third more
+// instructions, 96 registers): 185.
 // ===========================================================================
 constexpr int TT_M = 128;
 constexpr int TT_STAGES = 3;
 constexpr int TT_WORKERS = 8;                       // worker warps
+constexpr int TT_PF = 2;                            // A slices loaded ahead
+constexpr int TT_ACC = 4;                           // accumulators in TMEM (<= 4 x 128 columns)
+constexpr int TT_LAG = 2;                           // a slice is read out that many slices later
 constexpr int TT_THREADS = 32 * (TT_WORKERS + 1);   // + the control warp
 // TMEM columns of one accumulator (a power of two, at least 32)
 template <int NT>
@@ -455,7 +464,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     constexpr int CW = NT / G;                   // columns per worker thread
     constexpr int NCH = (CW + 31) / 32;          // 32-column TMEM loads per slice
     constexpr int OWNERS = 4 * G;                // worker warps holding columns
-    __shared__ uint64_t full_a[S], full_b[S], empty[S], accf[2], acce[2];
+    __shared__ uint64_t full_a[S], full_b[S], empty[S], accf[TT_ACC], acce[TT_ACC];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
 
@@ -464,14 +473,14 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     auto aborted = [&]() { return *(volatile int *)&abort_sh != 0; };
     // this CTA's work items: blockIdx.x + i gridDim.x; global slice g = i ns + s
     const int my_items = blockIdx.x < nitems ? (nitems - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const long total = (long)my_items * ns;
+    const int total = my_items * ns;
     if (tid == 0) {
         for (int b = 0; b < S; b++) {
             mbar_init(&full_a[b], TT_WORKERS);
             mbar_init(&full_b[b], 1);
             mbar_init(&empty[b], 1);
         }
-        for (int b = 0; b < 2; b++) {
+        for (int b = 0; b < TT_ACC; b++) {
             mbar_init(&accf[b], 1);
             mbar_init(&acce[b], OWNERS);
         }
@@ -481,19 +490,17 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_base_sh)),
-                     "r"(2 * TCOLS)
+                     "r"(TT_ACC * TCOLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base_sh;   // accumulator of slice g: columns (g & 1) TCOLS + ..
-    auto item_of = [&](long g, int &rb, int &ct) {
-        const int it = blockIdx.x + (int)(g / ns) * gridDim.x;
-        rb = it / P.ctiles;
-        ct = it % P.ctiles;
-    };
+    const uint32_t tmem = tmem_base_sh;   // accumulator of slice g: columns (g % TT_ACC) TCOLS + ..
+    // The roles walk their slices (slice of a work item, ring stage and its phase)
+    // by counters: divisions of a running slice number were most of the 630
+    // instructions a warp spent per slice.
     auto fail = [&]() {
         atomicExch(&abort_sh, 1);
         atomicOr(status, ST_TC_TIMEOUT);
@@ -503,40 +510,51 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
         // ----------------------------------------------------------------- control
         if (lane == 0) {
             const uint32_t idesc = idesc_tf32(TT_M, NT);
-            long b_issued = 0, b_landed = 0;
-            auto issue_b = [&](long g) {
-                int rb, ct;
-                item_of(g, rb, ct);
-                const unsigned char *src =
-                    image + ((size_t)ct * ns + (size_t)(g % ns)) * 2 * (size_t)BBYTES;
-                const int st = (int)(g % S);
-                unsigned char *dst = smem + st * STAGE + 2 * ABYTES;
-                mbar_expect_tx(&full_b[st], 2 * BBYTES);
-                bulk_g2s(dst, src, 2 * BBYTES, &full_b[st]);
+            int b_issued = 0, b_landed = 0;
+            // the next slice whose B half is copied
+            int bs = 0, bst = 0, bct = blockIdx.x % P.ctiles, bit = blockIdx.x;
+            auto issue_b = [&]() {
+                const unsigned char *src = image + ((size_t)bct * ns + bs) * 2 * (size_t)BBYTES;
+                mbar_expect_tx(&full_b[bst], 2 * BBYTES);
+                bulk_g2s(smem + bst * STAGE + 2 * ABYTES, src, 2 * BBYTES, &full_b[bst]);
                 b_issued++;
+                if (++bst == S) bst = 0;
+                if (++bs == ns) {
+                    bs = 0;
+                    bit += gridDim.x;
+                    bct = bit % P.ctiles;
+                }
             };
-            for (long g = 0; g < S - 1 && g < total; g++) issue_b(g);
-            for (long g = 0; g < total && !aborted(); g++) {
-                const int st = (int)(g % S);
-                const unsigned u = (unsigned)((g / S) & 1);
+            for (int g = 0; g < S - 1 && g < total; g++) issue_b();
+            int st = 0;
+            unsigned u = 0;
+            for (int g = 0; g < total && !aborted(); g++) {
                 if (!mbar_wait(&full_a[st], u) || !mbar_wait(&full_b[st], u)) { fail(); break; }
                 b_landed++;
-                // the accumulator of slice g - 2 has been read out
-                if (g >= 2 && !mbar_wait(&acce[g & 1], (unsigned)(((g - 2) >> 1) & 1))) { fail(); break; }
+                // the accumulator of slice g - TT_ACC has been read out
+                if (g >= TT_ACC && !mbar_wait(&acce[g % TT_ACC], (unsigned)((g / TT_ACC - 1) & 1))) {
+                    fail();
+                    break;
+                }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 unsigned char *base = smem + st * STAGE;
-                mma_slice_3xtf32(tmem + (uint32_t)((g & 1) * TCOLS), smem_u32(base),
+                mma_slice_3xtf32(tmem + (uint32_t)((g % TT_ACC) * TCOLS), smem_u32(base),
                                  smem_u32(base + ABYTES), smem_u32(base + 2 * ABYTES),
                                  smem_u32(base + 2 * ABYTES + BBYTES), idesc);
                 mma_commit(&empty[st]);
-                mma_commit(&accf[g & 1]);
+                mma_commit(&accf[g % TT_ACC]);
                 // the B half of stage (g - 1) % S is free once the MMAs of g - 1 are done
                 if (g + S - 1 < total) {
-                    if (g >= 1 && !mbar_wait(&empty[(g - 1) % S], (unsigned)(((g - 1) / S) & 1))) {
+                    const int pst = st == 0 ? S - 1 : st - 1;
+                    if (g >= 1 && !mbar_wait(&empty[pst], st == 0 ? u ^ 1u : u)) {
                         fail();
                         break;
                     }
-                    issue_b(g + S - 1);
+                    issue_b();
+                }
+                if (++st == S) {
+                    st = 0;
+                    u ^= 1u;
                 }
             }
             // B copies still in flight after an abort: wait for them (bounded)
@@ -556,24 +574,27 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
         float acc[NCH * 32];
 #pragma unroll
         for (int j = 0; j < NCH * 32; j++) acc[j] = 0.f;
-        float4 ra[AQ];
-        // A slice g into registers: chunk q = wt + 256 j: row q / 8, column quad (q % 8) * 4
-        auto load_a = [&](long g) {
-            int rb, ct;
-            item_of(g, rb, ct);
-            const long r0 = (long)rb * TT_M;
-            const int k0 = (int)(g % ns) * TC_K;
+        float4 ra[TT_PF][AQ];
+        // the thread's part of an A slice: column quad kq of rows row + RP j
+        constexpr int RP = 4 * TT_WORKERS;
+        const int row = wt >> 3, kq = (wt & 7) * 4;
+        const uint32_t aoff = sw128_offset(row, kq);   // + 128 RP j: RP a multiple of 8
+        int ls = 0, lit = blockIdx.x, lrb = lit / P.ctiles;   // the next slice to load
+        auto load_a = [&](float4 (&r)[AQ]) {
+            const int k = ls * TC_K + kq;
+            const long p0 = (long)lrb * TT_M + row;
+            if (vec4) {   // the quad lies in one of the blocks or beyond both
+                const bool first = k < P.k1, in = k < P.k1 + P.k2;
+                const int ld = first ? P.k1 : P.k2;
+                const float *src = first ? A1 + (size_t)p0 * ld + k : A2 + (size_t)p0 * ld + (k - P.k1);
 #pragma unroll
-            for (int j = 0; j < AQ; j++) {
-                const int q = wt + 32 * TT_WORKERS * j;
-                const int row = q >> 3, kq = (q & 7) * 4;
-                const long p = r0 + row;
-                const int k = k0 + kq;
-                if (p < P.n && vec4 && k + 3 < P.k1 + P.k2) {
-                    const float *src = k < P.k1 ? A1 + (size_t)p * P.k1 + k
-                                                : A2 + (size_t)p * P.k2 + (k - P.k1);
-                    ra[j] = *reinterpret_cast<const float4 *>(src);
-                } else {
+                for (int j = 0; j < AQ; j++)
+                    r[j] = in && p0 + RP * j < P.n ? *reinterpret_cast<const float4 *>(src + (size_t)(RP * j) * ld)
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+            } else {
+#pragma unroll
+                for (int j = 0; j < AQ; j++) {
+                    const long p = p0 + RP * j;
                     float v[4];
 #pragma unroll
                     for (int u = 0; u < 4; u++) {
@@ -582,26 +603,30 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
                         if (p < P.n && kk < P.k1) v[u] = A1[(size_t)p * P.k1 + kk];
                         else if (p < P.n && kk < P.k1 + P.k2) v[u] = A2[(size_t)p * P.k2 + (kk - P.k1)];
                     }
-                    ra[j] = make_float4(v[0], v[1], v[2], v[3]);
+                    r[j] = make_float4(v[0], v[1], v[2], v[3]);
                 }
+            }
+            if (++ls == ns) {
+                ls = 0;
+                lit += gridDim.x;
+                lrb = lit / P.ctiles;
             }
         };
         // the accumulator of slice h into registers, then release it
-        auto drain = [&](long h) -> bool {
+        auto drain = [&](int h) -> bool {
             if (!owner) return true;
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(&accf[h & 1], (unsigned)((h >> 1) & 1)));
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&accf[h % TT_ACC], (unsigned)((h / TT_ACC) & 1)));
             if (!ok) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            tmem_add32<NCH>(tl + (uint32_t)((h & 1) * TCOLS), acc);
+            tmem_add32<NCH>(tl + (uint32_t)((h % TT_ACC) * TCOLS), acc);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acce[h & 1]);
+            if (lane == 0) mbar_arrive(&acce[h % TT_ACC]);
             return true;
         };
-        // write out the finished work item of slice h, reset the sums
-        auto write_item = [&](long h) {
-            int rb, ct;
-            item_of(h, rb, ct);
+        // write out a finished work item, reset the sums
+        auto write_item = [&](int it) {
+            const int rb = it / P.ctiles, ct = it - rb * P.ctiles;
             double sq = 0.0;
             const long p = (long)rb * TT_M + wl + lane;
             if (owner && p < P.n) {
@@ -651,54 +676,64 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
                 if (lane == 0) part_sq[((size_t)rb * P.ctiles + ct) * TT_WORKERS + warp] = sq;
             }
         };
-        if (total > 0) load_a(0);
-        for (long g = 0; g < total; g++) {
-            const int st = (int)(g % S);
+        // slice h is read out; a work item ends with its last slice: write the item
+        int ds = 0, dit = blockIdx.x;
+        auto read_out = [&](int h) -> bool {
+            if (!drain(h)) return false;
+            if (++ds == ns) {
+                write_item(dit);
+                ds = 0;
+                dit += gridDim.x;
+            }
+            return true;
+        };
+        // one slice: split its values, load those of TT_PF slices on, read out the
+        // slice TT_LAG before; false: give up
+        int st = 0;   // ring stage
+        unsigned ph = 0;
+        auto slice = [&](int g, float4 (&r)[AQ]) -> bool {
             unsigned char *base = smem + st * STAGE;
             // the stage is free once the MMAs of slice g - S are done
-            if (g >= S && !__all_sync(0xffffffffu, mbar_wait(&empty[st], (unsigned)((g / S - 1) & 1)))) {
-                fail();
-                break;
-            }
-            if (aborted()) break;
+            if (g >= S && !__all_sync(0xffffffffu, mbar_wait(&empty[st], ph ^ 1u))) return false;
+            if (aborted()) return false;
 #pragma unroll
             for (int j = 0; j < AQ; j++) {
-                const int q = wt + 32 * TT_WORKERS * j;
-                const int row = q >> 3, kq = (q & 7) * 4;
-                const float v[4] = {ra[j].x, ra[j].y, ra[j].z, ra[j].w};
+                const float v[4] = {r[j].x, r[j].y, r[j].z, r[j].w};
                 float h[4], l[4];
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
                     h[u] = tf32_rna(v[u]);
                     l[u] = tf32_rna(v[u] - h[u]);
                 }
-                const uint32_t off = sw128_offset(row, kq);
-                *reinterpret_cast<float4 *>(base + off) = make_float4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<float4 *>(base + ABYTES + off) = make_float4(l[0], l[1], l[2], l[3]);
+                *reinterpret_cast<float4 *>(base + aoff + 128 * RP * j) = make_float4(h[0], h[1], h[2], h[3]);
+                *reinterpret_cast<float4 *>(base + ABYTES + aoff + 128 * RP * j) = make_float4(l[0], l[1], l[2], l[3]);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&full_a[st]);
-            if (g + 1 < total) load_a(g + 1);
-            // read out slice g - 1; a work item ends with it: write the item
-            if (g >= 1) {
-                if (!drain(g - 1)) {
-                    fail();
-                    break;
-                }
-                if ((g - 1) % ns == ns - 1) write_item(g - 1);
+            if (g + TT_PF < total) load_a(r);
+            if (++st == S) {
+                st = 0;
+                ph ^= 1u;
             }
-        }
-        if (total > 0 && !aborted()) {
-            if (drain(total - 1)) write_item(total - 1);
-            else fail();
-        }
+            return g < TT_LAG || read_out(g - TT_LAG);
+        };
+#pragma unroll
+        for (int u = 0; u < TT_PF; u++)
+            if (u < total) load_a(ra[u]);
+        bool ok = true;
+        for (int g = 0; ok && g < total; g += TT_PF)
+#pragma unroll
+            for (int u = 0; u < TT_PF; u++)
+                if (ok && g + u < total) ok = slice(g + u, ra[u]);
+        for (int h = max(0, total - TT_LAG); ok && h < total && !aborted(); h++) ok = read_out(h);
+        if (!ok && !aborted()) fail();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(2 * TCOLS)
+                     "r"(TT_ACC * TCOLS)
                      : "memory");
 }
 

@@ -60,9 +60,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
             : "r"(a), "r"(parity)
             : "memory");
         if (ok) return true;
-        if ((it & 1023u) == 0) {
+        // the timer from the 64th poll on: reading it after the first failed poll
+        // (most waits) costs more than the wait itself
+        if ((it & 63u) == 63u) {
             const unsigned long long t = tc_now_ns();
-            if (it == 0) t0 = t;
+            if (it == 63u) t0 = t;
             else if (t - t0 > 2000000000ull) return false;
         }
     }
