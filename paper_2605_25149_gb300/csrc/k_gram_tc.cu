@@ -275,22 +275,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                      : "memory");
 }
 
-// one thread per tile entry (grid: tiles x entry blocks), chunks summed in
-// order in FP64
-__global__ void k_gram_tc_reduce(TcPlan P, const float *partials, double w, double *out) {
-    const int tile = blockIdx.x;
+// CTA = 32 tile entries x 8 threads (grid: tiles x entry blocks), each summing an
+// eighth of the chunks in order in FP64, then the eighths in order: one thread per
+// entry waited for all the chunks' loads one after the other (64^3 points, 128
+// columns: 65 -> 27 us)
+__global__ void __launch_bounds__(256) k_gram_tc_reduce(TcPlan P, const float *partials, double w, double *out) {
+    __shared__ double red[8][33];
+    const int tile = blockIdx.x, g = threadIdx.y;
     int ta, tb;
     tc_tile_of(tile, P.tiles, ta, tb);
-    const int e = blockIdx.y * blockDim.x + threadIdx.x;
-    if (e >= TC_T * TC_T) return;
+    const int e = blockIdx.y * 32 + threadIdx.x;
     const int la = e / TC_T, lb = e % TC_T;
     const int a = ta * TC_T + la, b = tb * TC_T + lb;
-    if (a >= P.na || b >= P.na) return;
     // within a diagonal tile the MMA accumulates (i,j) and (j,i) in different
     // orders: keep the upper entry and mirror it
-    if (ta == tb && la > lb) return;
-    double s = ordered_sum(partials + (size_t)tile * TC_T * TC_T + e, P.chunks,
-                           (size_t)P.ntiles * TC_T * TC_T);
+    const bool ok = a < P.na && b < P.na && !(ta == tb && la > lb);
+    const int per = (P.chunks + 7) / 8, c0 = min(P.chunks, g * per), c1 = min(P.chunks, c0 + per);
+    const size_t stride = (size_t)P.ntiles * TC_T * TC_T;
+    red[g][threadIdx.x] =
+        ok ? ordered_sum(partials + (size_t)tile * TC_T * TC_T + e + c0 * stride, c1 - c0, stride) : 0.0;
+    __syncthreads();
+    if (g != 0 || !ok) return;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) s += red[k][threadIdx.x];
     s *= w;
     out[(size_t)a * P.na + b] = s;
     if (a != b) out[(size_t)b * P.na + a] = s;
@@ -326,7 +334,7 @@ void launch_gram_tc(long n, const float *X1, int n1, const float *X2, int n2, do
     tc_prepare();
     HQ_LAUNCH(HQ_K_GRAM, k_gram_tf32x3<<<dim3(p.ntiles, p.chunks), TC_THREADS, smem, s>>>(
                              p, X1, n1, X2, n2, partials, status));
-    HQ_LAUNCH(HQ_K_GRAM, k_gram_tc_reduce<<<dim3(p.ntiles, (TC_T * TC_T + 255) / 256), 256, 0, s>>>(
+    HQ_LAUNCH(HQ_K_GRAM, k_gram_tc_reduce<<<dim3(p.ntiles, TC_T * TC_T / 32), dim3(32, 8), 0, s>>>(
                              p, partials, w, out));
 }
 
