@@ -50,7 +50,9 @@ ALGO = {"smooth": (10.0, 3.0), "stencil": (10.0, 2.0), "residual": (9.0, 3.0)}
 #   z' = (omega c D^-1) s + ((1 - omega) z + rt): 5 add + 2 fma = 9 flops in 7
 #   FP64-pipe instructions; reads rt, z, writes z': 3 words
 ALGO_F64 = dict(ALGO, smooth=(9.0, 3.0))
-# FP64-pipe instructions per point-column (an add takes an issue slot as an FMA does)
+# FP64-pipe instructions per point-column of the kernels with FP64 additions (an
+# add takes an issue slot as an FMA does); the neighbour sums run on the integer
+# pipe, so fp64_issue_frac can exceed 1: the rate in units of that form's ceiling
 FP64_OPS = {"smooth": 7.0, "stencil": 8.0, "residual": 7.0}
 # DRAM bytes per point-column of the roofline kernels from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch / point-columns
