@@ -1076,10 +1076,43 @@ hq_status pcg(hq_ctx *x, const T *B, T *X, double rtol, int maxit, int *iters_ho
     return HQ_OK;
 }
 
+// The Gram plan of na x nb columns over the context's points, its split over the
+// points fitted to the workspace's partial sums: those are sized for the step's
+// 2N x 2N shapes, and a plan of fewer columns can have more tiles x chunks (N = 161:
+// 6 tiles x 50 chunks against 21 x 14), so then fewer, longer chunks.  False: one
+// chunk does not fit (not with na, nb <= 2N).
+bool gram_plan(const hq_ctx *x, int na, int nb, bool sym, GramPlan &gp) {
+    gp = make_gram_plan(x->n, na, nb, sym);
+    const size_t avail = std::max(gram_partial_bytes(x->gplan_max), gram_partial_bytes(x->gplan_uw));
+    if (gram_partial_bytes(gp) <= avail) return true;
+    const long max_chunks = (long)(avail / (gram_partial_bytes(gp) / gp.chunks));
+    if (max_chunks < 1) return false;
+    long rows = (x->n + max_chunks - 1) / max_chunks;
+    rows = (rows + 15) / 16 * 16;
+    gp.chunk_rows = rows;
+    gp.chunks = (int)((x->n + rows - 1) / rows);
+    return gram_partial_bytes(gp) <= avail;
+}
+
+// out = w [A1 A2]^T [B1 B2] by the SIMT Gram (sym: both triangles from the upper one)
+template <typename T>
+hq_status simt_gram(hq_ctx *x, const T *A1, int na1, const T *A2, int na2, const T *B1, int nb1, const T *B2,
+                    int nb2, bool sym, double w, double *out) {
+    GramPlan gp;
+    if (!gram_plan(x, na1 + na2, nb1 + nb2, sym, gp))
+        return fail(x, HQ_ERR_ARG, "Gram shape exceeds the workspace plan");
+    launch_gram<T>(gp, A1, na1, A2, na2, B1, nb1, B2, nb2, w, x->gpart, out, x->st);
+    return HQ_OK;
+}
+template <typename T>
+hq_status simt_gram(hq_ctx *x, const T *A, int na, const T *B, int nb, bool sym, double w, double *out) {
+    return simt_gram<T>(x, A, na, nullptr, 0, B, nb, nullptr, 0, sym, w, out);
+}
+
 // Symmetric Gram of [X1 X2] into out (FP64): SIMT FP64 in HQ_FP64 contexts,
 // tcgen05 3xTF32 in HQ_MIXED contexts.
 template <typename T>
-void gram_sym(hq_ctx *x, const T *X1, int n1, const T *X2, int n2, double *out);
+hq_status gram_sym(hq_ctx *x, const T *X1, int n1, const T *X2, int n2, double *out);
 // fp64_tc = 1 sends an FP64 product to the digit-sliced tensor-core kernels
 // only from this many multiply-adds on: below it their splitting passes and
 // one-CTA-per-SM schedule cost more than the SIMT FP64 kernels (a 4096 x 8
@@ -1090,18 +1123,18 @@ bool use_oz(const hq_ctx *x, double macs) {
 }
 
 template <>
-void gram_sym<double>(hq_ctx *x, const double *X1, int n1, const double *X2, int n2, double *out) {
+hq_status gram_sym<double>(hq_ctx *x, const double *X1, int n1, const double *X2, int n2, double *out) {
     const double na = n1 + n2;
     if (x->ozgram && gram_oz_supported(n1 + n2) && use_oz(x, 0.5 * (double)x->n * na * na)) {
         launch_gram_oz(x->n, X1, n1, X2, n2, x->h3, x->ozgram, out, x->status, x->st);
-        return;
+        return HQ_OK;
     }
-    GramPlan gp = make_gram_plan(x->n, n1 + n2, n1 + n2, true);
-    launch_gram<double>(gp, X1, n1, X2, n2, X1, n1, X2, n2, x->h3, x->gpart, out, x->st);
+    return simt_gram<double>(x, X1, n1, X2, n2, X1, n1, X2, n2, true, x->h3, out);
 }
 template <>
-void gram_sym<float>(hq_ctx *x, const float *X1, int n1, const float *X2, int n2, double *out) {
+hq_status gram_sym<float>(hq_ctx *x, const float *X1, int n1, const float *X2, int n2, double *out) {
     launch_gram_tc(x->n, X1, n1, X2, n2, x->h3, x->tcpart, out, x->status, x->st);
+    return HQ_OK;
 }
 
 // Out = A1 M1 (+ A2 M2) (+ Cin) (n x N); part_sq: sum of squares of Out into
@@ -1252,7 +1285,7 @@ hq_status enqueue_a(hq_ctx *x, StepGraph *sgr, long long *counters) {
     else HQ_CUDA(cudaMemsetAsync(W, 0, cnt * sizeof(T), x->st));
     if (sgr) HQ_TRY(pcg_device<T>(x, U, W, x->cfg.cg_rtol, x->cfg.cg_maxit, *sgr, counters));
     else HQ_TRY(pcg<T>(x, U, W, x->cfg.cg_rtol, x->cfg.cg_maxit, nullptr));
-    gram_sym<T>(x, U, N, W, N, x->G2);
+    HQ_TRY(gram_sym<T>(x, U, N, W, N, x->G2));
     // Msm = -Pwu (rows N..2N-1, columns 0..N-1 of G2); g = || W - U Pwu ||_h
     launch_extract(N, N, -1.0, x->G2 + (size_t)N * 2 * N, 2 * N, x->Msm, N, x->st);
     int np = 0;
@@ -1910,7 +1943,7 @@ hq_status set_initial_impl(hq_ctx *x, const double *U0, int on_device) {
     HQ_TRY(clear_status(x));
     T *U = (T *)x->U;
     HQ_TRY(load_block<T>(x, U, U0, on_device));
-    gram_sym<T>(x, U, N, (const T *)nullptr, 0, x->Ssm);
+    HQ_TRY(gram_sym<T>(x, U, N, (const T *)nullptr, 0, x->Ssm));
     launch_sym_eig(N, x->Ssm, x->eigwork, x->evals, nullptr, x->st);
     launch_inv_sqrt_first(x->evals, x->scal + 1, x->st);
     double lmin = 0;
@@ -2039,9 +2072,8 @@ hq_status eigen_impl(hq_ctx *x, double *evals_paper, double *evals_rr, double *e
     GridGeom g64 = make_geom(x->m, N, 8);
     launch_apply<double>(g64, v0.D, v0.c, U64, x->E2, nullptr, x->st);   // (H + sigma) U
     // <U, (H + sigma) U> is symmetric as <U,U> is: the upper tiles of both
-    GramPlan gs = make_gram_plan(x->n, N, N, true);
-    launch_gram<double>(gs, U64, N, nullptr, 0, x->E2, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
-    launch_gram<double>(gs, U64, N, nullptr, 0, U64, N, nullptr, 0, x->h3, x->gpart, x->Ssm, x->st);
+    HQ_TRY(simt_gram<double>(x, U64, N, x->E2, N, true, x->h3, x->Ksm));
+    HQ_TRY(simt_gram<double>(x, U64, N, U64, N, true, x->h3, x->Ssm));
     launch_axpy_small(N * N, -x->sigma, x->Ssm, x->Ksm, x->st);   // <U, H U>
     launch_rr_reduce(N, x->Ksm, x->Ssm, x->Lm, x->Cm, x->status, x->st);
     HQ_TRY(sync_status(x, x->status, "Rayleigh-Ritz (Cholesky of <U,U>)"));
@@ -2088,8 +2120,7 @@ hq_status monitor_impl(hq_ctx *x, double *energy, double *onorm, double *smin, d
     GridGeom g64 = make_geom(x->m, N, 8);
     // tr(U^T (H + sigma) U) as per-column partial dots, fused into the operator
     launch_apply<double>(g64, v0.D, v0.c, U64, x->E2, x->part, x->st);
-    GramPlan gs = make_gram_plan(x->n, N, N, true);
-    launch_gram<double>(gs, U64, N, nullptr, 0, U64, N, nullptr, 0, x->h3, x->gpart, x->Ssm, x->st);
+    HQ_TRY(simt_gram<double>(x, U64, N, U64, N, true, x->h3, x->Ssm));
     launch_monitor_finish(g64.gy * N, x->part, x->h3, N, x->Ssm, x->scal + 4, x->st);
     launch_sym_eig(N, x->Ssm, x->eigwork, x->evals, nullptr, x->st);
     double e2[2], ev_lo = 0, ev_hi = 0;
@@ -2167,8 +2198,7 @@ hq_status project(hq_ctx *x, double *y, double rtol = 0.0) {
         launch_gram_oz_xy(x->n, u, N, nullptr, 0, y, N, 2 * N, false, x->h3, x->ozgram, x->Ksm, x->status, x->st);
         launch_extract(N, N, -1.0, x->Ksm, N, x->Msm, N, x->st);
     } else {
-        GramPlan gp = make_gram_plan(x->n, N, N, false);
-        launch_gram<double>(gp, u, N, nullptr, 0, y, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
+        HQ_TRY(simt_gram<double>(x, u, N, y, N, false, x->h3, x->Ksm));
         launch_extract(N, N, -1.0, x->Ksm, N, x->Msm, N, x->st);
     }
     block_gemm<double>(x, u, N, x->Msm, nullptr, 0, nullptr, y, y, false, nullptr);
@@ -2354,9 +2384,8 @@ hq_status rayleigh_ritz_vectors(hq_ctx *x) {
     Level &v0 = x->lev[0];
     launch_apply<double>(v0.g, v0.D, v0.c, U64, x->E2, nullptr, x->st);   // (H + sigma) U
     // <U, (H + sigma) U> is symmetric as <U,U> is: the upper tiles of both
-    GramPlan gs = make_gram_plan(x->n, N, N, true);
-    launch_gram<double>(gs, U64, N, nullptr, 0, x->E2, N, nullptr, 0, x->h3, x->gpart, x->Ksm, x->st);
-    launch_gram<double>(gs, U64, N, nullptr, 0, U64, N, nullptr, 0, x->h3, x->gpart, x->Ssm, x->st);
+    HQ_TRY(simt_gram<double>(x, U64, N, x->E2, N, true, x->h3, x->Ksm));
+    HQ_TRY(simt_gram<double>(x, U64, N, U64, N, true, x->h3, x->Ssm));
     launch_axpy_small(N * N, -x->sigma, x->Ssm, x->Ksm, x->st);   // <U, H U>
     launch_rr_reduce(N, x->Ksm, x->Ssm, x->Lm, x->Cm, x->status, x->st);
     HQ_TRY(sync_status(x, x->status, "Rayleigh-Ritz (Cholesky of <U,U>)"));
@@ -2446,23 +2475,6 @@ hq_status pcg_impl(hq_ctx *x, const void *B, void *X, double rtol, int maxit, in
     HQ_TRY(clear_status(x));
     return pcg<T>(x, (const T *)B, (T *)X, rtol, maxit, iters);
 }
-// The split over grid points of a Gram must fit the workspace's partial sums
-// (sized for the step's own Gram shapes): otherwise fewer, longer point chunks.
-hq_status fit_gram_plan(hq_ctx *x, GramPlan &gp) {
-    const size_t avail = std::max(gram_partial_bytes(x->gplan_max), gram_partial_bytes(x->gplan_uw));
-    if (gram_partial_bytes(gp) <= avail) return HQ_OK;
-    const size_t per_chunk = sizeof(double) * (size_t)gp.ntiles * 64 * 64;
-    const long max_chunks = (long)(avail / per_chunk);
-    if (max_chunks < 1) return fail(x, HQ_ERR_ARG, "Gram shape exceeds the workspace plan");
-    long rows = (x->n + max_chunks - 1) / max_chunks;
-    rows = (rows + 15) / 16 * 16;
-    gp.chunk_rows = rows;
-    gp.chunks = (int)((x->n + rows - 1) / rows);
-    if (gram_partial_bytes(gp) > avail)
-        return fail(x, HQ_ERR_ARG, "Gram shape exceeds the workspace plan");
-    return HQ_OK;
-}
-
 // O'Leary's block PCG (not in the paper; an alternative to the per-column
 // recurrences of pcg()): X = G B with all N columns in one block Krylov space,
 // N x N step matrices alpha = (P^T Q)^-1 (Z^T R), beta = (Z^T R)^-1 (Z'^T R'):
@@ -2482,8 +2494,8 @@ hq_status coupled_pcg_impl(hq_ctx *x, const T *B, T *X, double rtol, int maxit, 
     Level &v = x->lev[0];
     const GridGeom &g = v.g;
     T *R = (T *)x->R, *Z = (T *)x->Zp, *P = (T *)x->P, *Q = (T *)x->Q, *Tt = (T *)x->Tt;
-    GramPlan gp = make_gram_plan(n, N, N, false);
-    HQ_TRY(fit_gram_plan(x, gp));
+    GramPlan gp;
+    if (!gram_plan(x, N, N, false, gp)) return fail(x, HQ_ERR_ARG, "Gram shape exceeds the workspace plan");
     auto inner = [&](const T *A, const T *Bm, double *out) {
         launch_gram<T>(gp, A, N, nullptr, 0, Bm, N, nullptr, 0, 1.0, x->gpart, out, x->st);
     };
@@ -2551,9 +2563,7 @@ hq_status gram_impl(hq_ctx *x, const void *A, int Na, const void *B, int Nb, dou
         HQ_TRY(check_launch(x));
         return sync_status(x, x->status, "tensor-core Gram");
     }
-    GramPlan gp = make_gram_plan(x->n, Na, Nb, A == B && Na == Nb);
-    HQ_TRY(fit_gram_plan(x, gp));
-    launch_gram<T>(gp, (const T *)A, Na, nullptr, 0, (const T *)B, Nb, nullptr, 0, w, x->gpart, out, x->st);
+    HQ_TRY(simt_gram<T>(x, (const T *)A, Na, (const T *)B, Nb, A == B && Na == Nb, w, out));
     return check_launch(x);
 }
 template <typename T>
