@@ -624,6 +624,11 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
     auto wait_done = [&](int q) -> bool {
         return mbar_wait(&done[q % OZ_GST], (unsigned)((q / OZ_GST) & 1));
     };
+    // TMEM is read by whole converged warps (tcgen05.ld.sync.aligned), so every
+    // exit from the slice loop is a decision of the warp, and the lanes that went
+    // their own ways (units without values, the issuing thread) meet again first.
+    auto warp_aborted = [&]() -> bool { return __any_sync(0xffffffffu, abort_sh); };
+    auto warp_done = [&](int q) -> bool { return __all_sync(0xffffffffu, wait_done(q)); };
     // fixed-point sums: thread = TMEM lane 32 (warp % 4) + lane (Gram row), 16
     // output columns (warp / 4)
     const int grow = (warp & 3) * 32 + lane, gcb = (warp >> 2) * 16;
@@ -631,6 +636,7 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
 #pragma unroll
     for (int j = 0; j < 16; j++) facc[j] = 0;
     auto flush = [&]() {
+        __syncwarp();
         oz_combine<OZ_GFRAC>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)gcb, facc, true);
     };
     // the MMAs of slice sl (one thread): digit i of the rows times up to four
@@ -695,11 +701,11 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
 #pragma unroll
         for (int k = 0; k < U; k++) load(0, k);
     for (int sl = 0; sl < nslices; sl++) {
-        if (abort_sh) break;
+        if (warp_aborted()) break;
         const int st = sl % OZ_GST;
         const bool fresh = sl % OZ_GFLUSH == 0;
         // the stage's previous slice is consumed
-        if (sl >= OZ_GST && !wait_done(sl - OZ_GST)) {
+        if (sl >= OZ_GST && !warp_done(sl - OZ_GST)) {
             abort_sh = 1;
             break;
         }
@@ -724,7 +730,7 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
         mbar_arrive(&full[st]);
         if (fresh && sl > 0) {
             // 128 points accumulated: every MMA so far is complete
-            if (!wait_done(sl - 1)) {
+            if (!warp_done(sl - 1)) {
                 abort_sh = 1;
                 break;
             }
@@ -742,6 +748,7 @@ __global__ void __launch_bounds__(OZ_GTHREADS, 1)
                 issue(sl, fresh);
             }
         }
+        __syncwarp();
     }
     if (!abort_sh && nslices > 0 && !wait_done(nslices - 1)) abort_sh = 1;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
