@@ -695,6 +695,8 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
             }
             return true;
         };
+        // giving up is a decision of the warp: read_out's TMEM loads take all its lanes
+        auto warp_aborted = [&]() -> bool { return __any_sync(0xffffffffu, aborted()); };
         // one slice: split its values, load those of TT_PF slices on, read out the
         // slice TT_LAG before; false: give up
         int st = 0;   // ring stage
@@ -703,7 +705,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
             unsigned char *base = smem + st * STAGE;
             // the stage is free once the MMAs of slice g - S are done
             if (g >= S && !__all_sync(0xffffffffu, mbar_wait(&empty[st], ph ^ 1u))) return false;
-            if (aborted()) return false;
+            if (warp_aborted()) return false;
 #pragma unroll
             for (int j = 0; j < AQ; j++) {
                 const float v[4] = {r[j].x, r[j].y, r[j].z, r[j].w};
@@ -734,7 +736,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
 #pragma unroll
             for (int u = 0; u < TT_PF; u++)
                 if (ok && g + u < total) ok = slice(g + u, ra[u]);
-        for (int h = max(0, total - TT_LAG); ok && h < total && !aborted(); h++) ok = read_out(h);
+        for (int h = max(0, total - TT_LAG); ok && h < total && !warp_aborted(); h++) ok = read_out(h);
         if (!ok && !aborted()) fail();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
