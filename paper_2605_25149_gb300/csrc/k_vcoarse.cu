@@ -713,6 +713,10 @@ size_t vcoarse_smem_bytes(const VCoarse &v) {
     return vc_floats(v) * sizeof(float) + 8 * sizeof(double) * (size_t)v.nc;
 }
 
+bool vcoarse_fits(const VCoarse &v) {
+    return v.m[0] <= VC_MAX_SIDE && vcoarse_smem_bytes(v) <= (size_t)VC_MAX_SMEM;
+}
+
 size_t vcoarse64_smem_bytes(const VCoarse &v, const GridGeom &g64) {
     return vcoarse_smem_bytes(v) + sizeof(double) * (size_t)g64.gy * g64.ty;
 }
