@@ -721,7 +721,7 @@ int fuse_level(const hq_ctx *x, bool honour_switch = true) {
     if (x->nc > 64) return -1;   // k_vcoarse's coarsest solve: at most 64 points (4^3)
     for (int l = 0; l + 1 < x->L; l++) {
         if (x->L - l > VC_MAXLEV) continue;
-        if (vcoarse_fits(make_vcoarse(x, l))) return l;
+        if (vcoarse_smem_bytes(make_vcoarse(x, l)) <= (size_t)VC_MAX_SMEM) return l;
     }
     return -1;
 }
@@ -2735,6 +2735,7 @@ hq_status hq_init(const hq_config *cfg, void *d_workspace, size_t bytes, void *c
     if (x->mixed) hq::tc_prepare();
     hq::lu_prepare();
     hq::vcoarse_prepare();
+    hq::pcg_small_prepare();
     hq::rows_prepare();
     hq::lu32_prepare();
     hq::sym_eig_prepare();

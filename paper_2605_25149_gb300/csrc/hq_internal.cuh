@@ -176,14 +176,13 @@ void launch_dot(const GridGeom &g, const T *x, const T *y, double *part, cudaStr
 // one CTA per column, every level's vectors in shared memory.  Arrays are
 // indexed from l0 (entry 0 = level l0); the last entry is the coarsest level.
 constexpr int VC_MAXLEV = 8;
-constexpr int VC_MAX_SMEM = 226 * 1024;
-// The largest side that starts such a launch.  20^3 and its coarser levels would fit
-// too (229,752 bytes), but as separate kernels with the FP64 interface in the PCG's
-// passes they are faster at every width: 15 PCG iterations at 20^3, FP32
-// preconditioner, 1 column 1197 against 1065 us (one launch, separate), 8 columns
-// 1219, 1054, 64 columns 1639, 1394, 152 columns 2037, 1967, 256 columns 3216, 2687;
-// with 20^3 as the second level (40^3, 64 columns) 4119, 3833.
-constexpr int VC_MAX_SIDE = 19;
+// 19^3 and its coarser levels take 178 KB.  20^3 (208,552 bytes) would fit an SM, but
+// as separate kernels with the FP64 interface in the PCG's passes it is faster at
+// every width: 15 PCG iterations at 20^3, FP32 preconditioner, 1 column 1197 against
+// 1065 us (one launch, separate), 8 columns 1219, 1054, 64 columns 1639, 1394, 152
+// columns 2037, 1967, 256 columns 3216, 2687; with 20^3 as the second level (40^3, 64
+// columns) 4119, 3833.
+constexpr int VC_MAX_SMEM = 200 * 1024;
 struct VCoarse {
     int levels;                       // levels in the launch (>= 2)
     int m[VC_MAXLEV];                 // nodes per side
@@ -200,7 +199,6 @@ struct VCoarse {
     int nu1, nu2;
 };
 size_t vcoarse_smem_bytes(const VCoarse &v);
-bool vcoarse_fits(const VCoarse &v);
 // sets the dynamic shared-memory limit (call once, outside any stream capture)
 void vcoarse_prepare();
 // z = V-cycle(r) from level l0 for all N columns (point-major n_l0 x N FP32 blocks)
@@ -220,6 +218,8 @@ void launch_vcoarse64(const VCoarse &v, const GridGeom &g64, const double *r64, 
 // num_active[1] (iterations of the slowest column), which counters[0]
 // (nullable) receives too; ST_PCG_MAXIT at the cap when check_maxit.
 bool pcg_small_fits(const VCoarse &v, const GridGeom &g);
+// sets the dynamic shared-memory limit (call once, outside any stream capture)
+void pcg_small_prepare();
 void launch_pcg_small(const VCoarse &v, const GridGeom &g, const double *D64, double c64, const double *B,
                       double *X, const PcgScalars &sc, double rtol, int maxit, long long *counters,
                       int check_maxit, cudaStream_t s);
