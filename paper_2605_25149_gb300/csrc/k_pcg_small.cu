@@ -603,8 +603,13 @@ size_t ps_smem_bytes(const VCoarse &v, const GridGeom &g) {
 
 }  // namespace
 
+// One CTA per column and SM: a second wave of columns still beats the separate
+// kernels up to 16^3 (to rounding there), a third nowhere.  15 iterations, one launch
+// against separate kernels: 160 columns 8^3 870, 994 us, 13^3 1474, 1514, 16^3 1920, 1915, 17^3
+// 2205, 2055; 320 columns 8^3 1280, 1108, 13^3 2186, 1916, 16^3 2636, 2441.
 bool pcg_small_fits(const VCoarse &v, const GridGeom &g) {
     const long n = (long)v.m[0] * v.m[0] * v.m[0];
+    if (g.N > (n <= 4096 ? 2 : 1) * 152) return false;
     return v.levels >= 2 && n <= (long)PS_U * VC_THREADS && (long)g.gy * g.ty <= (long)PS_U * VC_THREADS &&
            (g.gy + 127) / 128 <= VC_THREADS / 8 && ps_smem_bytes(v, g) <= (size_t)PS_MAX_SMEM;
 }

@@ -24,6 +24,14 @@ def test_finest_level_of_an_fp32_preconditioner(m, separate):
     assert (la["smooth"] > 0) == separate, la
 
 
+@pytest.mark.parametrize("m,N,one", [(8, 152, True), (16, 304, True), (16, 305, False), (17, 152, True),
+                                     (17, 153, False), (18, 4, False)])
+def test_one_launch_pcg_by_waves_of_columns(m, N, one):
+    """One CTA per column: two waves of the 152 SMs up to 16^3 points, one at 17^3."""
+    la = launches(m, N, mg_fp32=1)
+    assert (la["stencil"] == 0) == one, la
+
+
 @pytest.mark.parametrize("m,separate", [(38, False), (39, False), (40, True), (41, True)])
 @pytest.mark.parametrize("kw", [dict(mg_fp32=1), dict(precision="mixed", cg_rtol=1e-6)])
 def test_second_level(m, separate, kw):
