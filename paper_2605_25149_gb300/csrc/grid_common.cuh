@@ -78,9 +78,15 @@ __device__ __forceinline__ double sum6_aligned(const unsigned (&hi)[6], const un
 static __device__ __noinline__ double sum6_scaled(double a0, double a1, double a2, double a3, double a4,
                                            double a5) {
     double a[6] = {a0, a1, a2, a3, a4, a5};
-    unsigned hi[6], lo[6], ex[6], E = 0;
+    unsigned hi[6], lo[6], ex[6], E = 0, any = 0;
 #pragma unroll
-    for (int k = 0; k < 6; k++) E = max(E, ((unsigned)__double2hiint(a[k]) << 1) >> 21);
+    for (int k = 0; k < 6; k++) {
+        E = max(E, ((unsigned)__double2hiint(a[k]) << 1) >> 21);
+        any |= ((unsigned)__double2hiint(a[k]) << 1) | (unsigned)__double2loint(a[k]);
+    }
+    // six zeros, the first residual of a solve from zero: the scaling's products on
+    // the FP64 pipe made it the slowest case of all (64^3, 64 columns 478 us)
+    if (any == 0) return 0.0;
     if (E == 2047u) return ((a0 + a1) + (a2 + a3)) + (a4 + a5);
     const bool low = E < 64u;
     E = 0;
@@ -92,7 +98,6 @@ static __device__ __noinline__ double sum6_scaled(double a0, double a1, double a
         ex[k] = (hi[k] << 1) >> 21;
         E = max(E, ex[k]);
     }
-    if (E == 0) return 0.0;   // six zeros
     return sum6_aligned(hi, lo, ex, E) * (low ? 0x1p-128 : 0x1p128);
 }
 __device__ __forceinline__ double sum6(const double (&a)[6], const bool (&in)[6]) {
