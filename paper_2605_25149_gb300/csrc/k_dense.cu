@@ -1491,7 +1491,7 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
     }
 }
 
-// The same eigenproblem for N <= SE_MAX in three parts, since one SM's FP64
+// The same eigenproblem for SE_MIN <= N <= SE_MAX in three parts, since one SM's FP64
 // rate (about 2.3 lanes per clock) bounds cyclic Jacobi: an FP64 sweep of N = 64
 // with vectors takes 0.27 ms in shared memory and eight or nine are needed.
 //  1. FP32 Jacobi of A scaled by a power of two (k_sym_eig_sm<float>): V0, whose
@@ -1504,6 +1504,8 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
 // FP64 Jacobi with the tolerance of k_sym_eig whatever V0 was.
 // Measured, N = 64: 7 ms in one FP64 launch before; now 0.6 + 0.08 + 0.66 ms (0.08 ms
 // for part 1 where A is nearly diagonal, as in every refinement round but the first).
+constexpr int SE_MIN = 5;   // below, the seven launches cost more than the one above: an initial block of 8^3
+                            // points, 1 column 127 against 86 us, 4 columns 161, 145, 5 columns 166, 169
 constexpr int SE_MAX = 112;
 constexpr int SE_THREADS = 1024;
 constexpr int SE_BLK = (SE_MAX / 2 * (SE_MAX / 2 - 1) / 2 + SE_THREADS - 1) / SE_THREADS;
@@ -1743,12 +1745,12 @@ void sym_eig_prepare() {
 
 size_t sym_eig_work_doubles(int N) {
     const size_t P2 = (size_t)((N + 1) & ~1) * ((N + 1) & ~1);
-    return N <= SE_MAX ? 5 * (size_t)N * N + 1 : 2 * P2;
+    return N >= SE_MIN && N <= SE_MAX ? 5 * (size_t)N * N + 1 : 2 * P2;
 }
 
 void launch_sym_eig(int N, const double *A, double *work, double *evals, double *evecs,
                     cudaStream_t s) {
-    if (N <= SE_MAX) {
+    if (N >= SE_MIN && N <= SE_MAX) {
         const size_t NN = (size_t)N * N;
         double *V = work, *G = work + NN, *M = work + 2 * NN, *V1 = work + 3 * NN, *As = work + 4 * NN,
                *scale = work + 5 * NN;
