@@ -6,6 +6,7 @@
 #include "hq_internal.cuh"
 
 #include <algorithm>
+#include <climits>
 
 namespace hq {
 
@@ -1495,7 +1496,8 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
 // rate (about 2.3 lanes per clock) bounds cyclic Jacobi: an FP64 sweep of N = 64
 // with vectors takes 0.27 ms in shared memory and eight or nine are needed.
 //  1. FP32 Jacobi of A scaled by a power of two (k_sym_eig_sm<float>): V0, whose
-//     columns diagonalise A to 1e-6 of its norm (its rounding floor is near 4e-7);
+//     columns diagonalise A to 1e-6 of its norm (its rounding floor is near 4e-7)
+//     and to 1e-4 beside its diagonal entries;
 //  2. V1 = V0 (15/8 I - 10/8 G + 3/8 G^2), G = V0^T V0: orthogonal to FP64
 //     rounding (the step cubes V0's 1e-6), and A' = V1^T A V1 in FP64 on many CTAs;
 //  3. FP64 Jacobi of A' continuing V1 (k_sym_eig_sm<double>): the off-diagonal
@@ -1510,16 +1512,34 @@ constexpr int SE_MAX = 112;
 constexpr int SE_THREADS = 1024;
 constexpr int SE_BLK = (SE_MAX / 2 * (SE_MAX / 2 - 1) / 2 + SE_THREADS - 1) / SE_THREADS;
 
+// 2^-e of 2^e <= x < 2^(e+1) (x normal, e < 1023 or 127)
+__device__ __forceinline__ double inverse_binade(double x) {
+    return __hiloint2double(0x7fe00000 - (__double2hiint(x) & 0x7ff00000), 0);
+}
+__device__ __forceinline__ float inverse_binade(float x) {
+    return __int_as_float(0x7f000000 - (__float_as_int(x) & 0x7f800000));
+}
+
 // One-CTA cyclic Jacobi in shared memory, round-robin pairs, the rotations of a
 // round applied to the 2 x 2 blocks of all pairs of pairs at once (each block
 // once, its mirror image written with it).  The tangent of each rotation is
 // formed in FP32 (an inexact angle leaves 1e-7 of the element, which later
 // sweeps remove), its cosine from that tangent to the working precision, so the
-// rotations are orthogonal to rounding.  Elements at or below `skip` are left.
+// rotations are orthogonal to rounding.  Elements at or below `skip` that are also
+// small beside their diagonal entries (|a_pq| <= rskip sqrt|a_pp a_qq|) are left.
+//
+// The sweeps end with the off-diagonal below `tol`, and up to four sweeps later
+// when no element exceeds rtol sqrt|a_pp a_qq| or their count no longer falls: the
+// small eigenvalues of a graded matrix (columns of very different norms) keep their
+// relative accuracy only so.  With `tol` alone the smallest one of a Gram of columns
+// scaled over seven orders had errors of 1e-8 to 6e-7 (1e-14 in one FP64 launch); now
+// below 1e-14.  Ordinary spectra meet both at once (one sweep more with an eigenvalue
+// near zero).
 template <typename T>
 __device__ void jacobi_sweeps(int P, int N, T *A, T *V, T *cs, T *sn, int *pp, int *qq, T *red, T tol,
-                              T skip, int max_sweeps) {
+                              T skip, T rtol, T rskip, int max_sweeps) {
     const int tid = threadIdx.x, LD = P + 1, H = P / 2;
+    int large = INT_MAX, extra = 0;   // threads that saw an element above rtol; sweeps behind tol
     const int blocks = H * (H - 1) / 2;   // at most SE_BLK per thread
     // blocks of different pairs: (k, k + d mod H), decoded once
     int bk[SE_BLK], bl[SE_BLK];
@@ -1537,19 +1557,27 @@ __device__ void jacobi_sweeps(int P, int N, T *A, T *V, T *cs, T *sn, int *pp, i
     const int warp = tid >> 5, lane = tid & 31;
     for (int sweep = 0; sweep < max_sweeps; sweep++) {
         T off = T(0);
+        bool above = false;
         for (int idx = tid; idx < P * P; idx += SE_THREADS) {
             const int i = idx / P, j = idx - i * P;
-            if (i < j) off += A[i * LD + j] * A[i * LD + j];
+            if (i >= j) continue;
+            const T a2 = A[i * LD + j] * A[i * LD + j];
+            off += a2;
+            above = above || a2 > rtol * rtol * fabs(A[i * LD + i] * A[j * LD + j]);
         }
         red[tid] = off;
-        __syncthreads();
+        const int now = __syncthreads_count(above);
         for (int w = SE_THREADS / 2; w > 0; w >>= 1) {
             if (tid < w) red[tid] += red[tid + w];
             __syncthreads();
         }
         off = red[0];
         __syncthreads();
-        if (sqrt(off) <= tol || off == T(0)) break;
+        if (sqrt(off) <= tol || off == T(0)) {
+            if (now == 0 || now >= large || extra == 4) break;
+            large = now;
+            extra++;
+        }
         for (int r = 0; r < P - 1; r++) {
             if (tid < H) {
                 int a = P - 1, b = r;
@@ -1563,9 +1591,11 @@ __device__ void jacobi_sweeps(int P, int N, T *A, T *V, T *cs, T *sn, int *pp, i
                 pp[tid] = p;
                 qq[tid] = q;
                 T c = T(1), sv = T(0);
-                const T apq = A[p * LD + q];
-                if (fabs(apq) > skip) {
-                    const float x = (float)(A[q * LD + q] - A[p * LD + p]), y = 2.f * (float)apq;
+                const T apq = A[p * LD + q], app = A[p * LD + p], aqq = A[q * LD + q];
+                if (fabs(apq) > skip || apq * apq > rskip * rskip * fabs(app * aqq)) {
+                    // scaled by a power of two: the squares of small entries stay in range
+                    const T dx = aqq - app, dy = T(2) * apq, sc = inverse_binade(fmax(fabs(dx), fabs(dy)));
+                    const float x = (float)(dx * sc), y = (float)(dy * sc);
                     const float t = (x >= 0.f ? y : -y) / (fabsf(x) + sqrtf(x * x + y * y));
                     const T u = T(1) + (T)t * (T)t;
                     c = (T)rsqrtf((float)u);
@@ -1689,7 +1719,8 @@ __global__ void __launch_bounds__(SE_THREADS) k_sym_eig_sm(int N, const double *
     __syncthreads();
     // skipped elements together stay below the tolerance: P^2/2 of them at most
     const T tol = (F32 ? T(1e-6) : T(1e-15)) * fro;
-    jacobi_sweeps<T>(P, N, A, V, cs, sn, pp, qq, red, tol, tol / (T)(2 * P), F32 ? 12 : 100);
+    jacobi_sweeps<T>(P, N, A, V, cs, sn, pp, qq, red, tol, tol / (T)(2 * P), F32 ? T(1e-4) : T(1e-14),
+                     F32 ? T(1e-5) : T(2e-16), F32 ? 16 : 100);
     if (F32) {
         __shared__ int bad;
         if (tid == 0) bad = 0;
