@@ -38,9 +38,10 @@ __device__ __forceinline__ float sum6(const float (&x)[6], const bool (&in)[6]) 
 // clocks per sum).  The terms are aligned to the largest
 // exponent E of the six as 60-bit magnitudes (7 guard bits below the 53 of
 // the largest term), added in 64 bits and rounded once: the error is at most
-// 6 truncations of 2^-59 2^E and one rounding of the result, below that of
-// five rounded additions, whatever their order; the sum is an odd,
-// order-independent function of its terms.  Terms with E outside [64, 2040]
+// 6 truncations of 2^-59 2^E and one rounding of the result.  That is an absolute
+// bound, relative to the largest term: where larger terms cancel exactly, what lies 59
+// binades below them is lost, which additions in a lucky order would have kept.  The
+// sum is an odd, order-independent function of its terms.  Terms with E outside [64, 2040]
 // (subnormal or near overflow) are scaled by a power of two first; an infinity
 // or a NaN among them takes the plain additions.
 // hi, lo, ex: the words and biased exponents of the six values, E: the largest

@@ -6,15 +6,15 @@
 // GB300 retires about two FP64 lane operations per clock per SM, so the FP64
 // SIMT form of these products is bound by the FP64 pipe.  Here every value is
 // written as a scaled sum of 7 balanced base-256 digits,
-//   A[p][k] = 2^(e_p + 1) sum_{i=1..7} a_i 2^(-8i)   (+- 2^-56 |row max|, rounded),
-// with e_p taken from the largest exponent of row p (points) of [A1 A2], and
-// likewise for each column c of [M1; M2].  Digits are integers -128..128, exact
-// in fp16.  Products of digit pairs with the same i + j = t share the scale
-// 2^(-8t) and are accumulated by kind::f16 MMAs into one FP32 TMEM
-// accumulator D_t; every partial sum is an integer of at most
+//   A[p][k] = 2^(e_p + 1) sum_{i=1..7} a_i 2^(-8i)   (+- 2^-55 |row max|, rounded),
+// with e_p taken from the largest exponent of row p (points) of [A1 A2], 2^(e_p - 1) <=
+// |row max| < 2^e_p, and likewise for each column c of [M1; M2].  Digits are integers
+// -128..128, exact in fp16.  Products of digit pairs with the same i + j = t share the
+// scale 2^(-8t) and are accumulated by kind::f16 MMAs into one FP32 TMEM accumulator D_t; every partial sum is an integer of at most
 // 7 * K * 128^2 < 2^24 for K <= 128, so the accumulation is exact.  Pairs with
-// t <= 8 are kept (the dropped ones are below 2^-53 of |row max| |column max|
-// per term).  The epilogue combines D_2..D_8 in 64-bit fixed point, converts
+// t <= 8 are kept (the dropped ones, six of t = 9 first, are below 2^-51 of |row max|
+// |column max| per term: 6 128^2 2^-72 2^(e_p + f_c + 2); digits 65, -128, .., -128 on both
+// sides come to 2^-51.4).  The epilogue combines D_2..D_8 in 64-bit fixed point, converts
 // once to FP64, applies 2^(e_p + f_c), adds Cin and optionally sums squares.
 // (Eight 7-bit sign-magnitude digits in bf16 have the same bounds but 36 digit
 // products instead of 28, and took 3.5 instead of 1.3 instructions per digit
@@ -514,7 +514,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // (36 products of 7-bit digits as MMAs of 64 columns; the same digits with this
 // schedule: 215).  The exact-sum bound holds for 128 points, so every four
 // slices the seven accumulators are read and added into 64-bit fixed-point
-// registers (OZ_GFRAC fraction bits); the chunk's FP64 partial tile is
+// registers (OZ_GFRAC fraction bits, the rest truncated: below 2^-44 of |x max| |y max|
+// per read-out); the chunk's FP64 partial tile is
 // summed over chunks in a fixed order by k_oz_gram_reduce.  D_t(i,j) and
 // D_t(j,i) are the same integers, so <X, X> is exactly symmetric.
 // ---------------------------------------------------------------------------
