@@ -392,14 +392,17 @@ RowShape row_shape(int len, int N) {
 // steps per CTA of a march of `len` steps: about 16 CTAs per SM (2 to 16 per SM
 // measured: 64^3, 64 columns 320, 301, 294, 299 us per V-cycle, 96^3 925, 871, 854,
 // 834 us, 128^3 within 2%) but at least four steps; fewer where even so the CTAs
-// do not fill four per SM (a step waits for its loads, so on small levels the
-// march itself was the time: y/z-restriction of 16^3, 32 columns 16 us)
-int march_chunk(long ctas, int len) {
+// do not fill `few` per SM (a step waits for its loads, so on small levels the
+// march itself was the time: y/z-restriction of 16^3, 32 columns 16 us).  Four,
+// but two for the FP64 y/z-restriction: a chunk forms the y-taps of the fine planes it
+// shares with the next one again, on the FP64 pipe (restriction from 20^3, 256 columns
+// 39.6 -> 33.6 us, 64^3, 8 columns 38.8 -> 33.6; 35.7 and 35.7 as three passes).
+int march_chunk(long ctas, int len, long few = 4) {
     auto chunk = [&](long target) {
         const long ch = std::max(1L, std::min((long)len, (target + ctas - 1) / ctas));
         return (int)((len + ch - 1) / ch);
     };
-    return std::max(chunk(152L * 16), std::min(4, chunk(152L * 4)));
+    return std::max(chunk(152L * 16), std::min(4, chunk(152L * few)));
 }
 template <typename T>
 size_t row_smem_bytes(const RowShape &s, int m, int mc) {
@@ -431,7 +434,7 @@ template <typename T, int V>
 void run_restrict_yz(const RowShape &s, int mf, int mc, int N, const XferTab &t, T scale, const T *in,
                      T *out, cudaStream_t st) {
     const int ty = std::max(1, 256 / s.lx), gy = (mc * mc + ty - 1) / ty;
-    const int cz = march_chunk((long)s.gx * gy, mc);
+    const int cz = march_chunk((long)s.gx * gy, mc, sizeof(T) == 8 ? 2 : 4);
     HQ_LAUNCH_W(HQ_K_TRANSFER, (double)mc * mc * mc * N,
                 k_restrict_yz<T, V><<<dim3(s.gx, gy, (mc + cz - 1) / cz), dim3(s.lx, ty), 0, st>>>(
                     mf, mc, N, cz, t.ridx, taps<T>(t.rw, t.rwf), taps<T>(t.pw, t.pwf), scale, in, out));
