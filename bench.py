@@ -54,12 +54,17 @@ ALGO_F64 = dict(ALGO, smooth=(9.0, 3.0))
 # add takes an issue slot as an FMA does); the neighbour sums run on the integer
 # pipe, so fp64_issue_frac can exceed 1: the rate in units of that form's ceiling
 FP64_OPS = {"smooth": 7.0, "stencil": 8.0, "residual": 7.0}
+# Integer-ALU lane instructions per point-column of the FP64 grid kernels, which
+# bound them (sm__inst_executed_pipe_alu.sum x 32 / point-columns of one ncu capture
+# at 64^3, N = 64), and the pipe's rate: 64 lanes / clk / SM x 152 SMs x 2.07 GHz
+INT_OPS = {"smooth": 54337536 * 32 / 16777216, "stencil": 56713216 * 32 / 16777216}
+INT_PEAK_TOPS = 64 * 152 * 2.07e9 / 1e12
 # DRAM bytes per point-column of the roofline kernels from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch / point-columns
 # of that launch): keys (class, dtype); an entry is removed whenever its
 # kernel changes, until it is captured again.
 TRAFFIC_PER_ELEMENT = {("smooth", "f32"): (136.215040e6 + 44.029440e6) / 16777216,
-                       ("stencil", "f64"): (136.446208e6 + 96.011008e6) / 16777216,
+                       ("stencil", "f64"): (136.435968e6 + 95.227392e6) / 16777216,
                        # the z-marching FP32 sweep (blocks of 100 MB or more),
                        # captured on 64^3 x 256 and scaled by point-columns
                        ("smooth_zm", "f32"): (553.649408e6 + 240.579328e6) / 67108864}
@@ -271,6 +276,20 @@ def roofline_alone(kind, ms_launch, n_el, dtype_tag, hbm_peak, hbm_kind, in_step
         out.update({"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak, "peak_source": hbm_kind})
     out["in_step"] = in_step
+    return out
+
+
+def integer_roof(entry, kind):
+    """An FP64 grid kernel's entry against the pipe that bounds it, the integer
+    ALU (the neighbour sums run there); the FP64 figures move below "fp64_pipe"."""
+    keys = ("achieved", "peak", "unit", "frac", "peak_source", "fp64_issue_frac")
+    out = dict(entry, fp64_pipe={k: entry[k] for k in keys})
+    out.pop("fp64_issue_frac")
+    achieved = INT_OPS[kind] * entry["elements_per_launch"] / (entry["ms_per_launch"] / 1e3) / 1e12
+    out.update({"achieved": achieved, "peak": INT_PEAK_TOPS, "unit": "Tinstr/s (integer ALU lanes)",
+                "frac": achieved / INT_PEAK_TOPS,
+                "peak_source": "derived: 64 integer-ALU lanes/clk/SM x 152 SMs x 2.07 GHz; instructions "
+                               "per point-column from an ncu capture"})
     return out
 
 
@@ -991,6 +1010,8 @@ def run_hq(args):
     kind = "stencil" if w.get("mg_fp32") else dominant(prof)
     roof = roofline_alone(kind, kernel_alone(torch, s, kind, not w.get("mg_fp32")), m ** 3 * N,
                           "f64", hbm_peak, hbm_kind, roofline(prof, kind, "f64"))
+    if kind in INT_OPS:
+        roof = integer_roof(roof, kind)
     brk = breakdown(prof, K)
     # end to end through host buffers: state in from pinned host memory,
     # step, state and gradient norm back to pinned host memory

@@ -356,7 +356,8 @@ typedef enum {
     HQ_K_SMOOTH,        /* damped-Jacobi sweeps                            */
     HQ_K_TRANSFER,      /* restriction / prolongation                      */
     HQ_K_COARSE,        /* coarsest-level solve, or the coarse levels of an */
-                        /* FP32 V-cycle in one launch                      */
+                        /* FP32 V-cycle in one launch, or a whole inner     */
+                        /* solve in one launch (FP64, mg_fp32, 17^3 at most) */
     HQ_K_VECTOR,        /* PCG vector updates, dots, conversions           */
     HQ_K_REDUCE,        /* per-column / global finalising reductions       */
     HQ_K_GRAM,          /* inner-product matrices <A,B>                    */

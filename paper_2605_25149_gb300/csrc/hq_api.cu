@@ -126,7 +126,7 @@ struct hq_ctx {
     float *tcpart = nullptr;   // tensor-core Gram partials (HQ_MIXED)
     unsigned char *tcimg = nullptr;   // split small matrix of the tensor-core block products
     TallPlan tplan;
-    double *tpart = nullptr;   // gy x N
+    double *tpart = nullptr;   // block-product partials
     double *G2 = nullptr, *Mw = nullptr, *XY = nullptr, *C = nullptr, *T1 = nullptr;
     double *Shat = nullptr, *Om = nullptr, *Msm = nullptr, *Ksm = nullptr, *Ssm = nullptr;
     double *Lm = nullptr, *Cm = nullptr, *Ym = nullptr, *Cv = nullptr;
@@ -453,8 +453,8 @@ size_t carve(hq_ctx *x, const hq_config *c, char *base) {
     GramPlan gmax = make_gram_plan(n, 2 * N, 2 * N, false);
     double *gpart = cv.take<double>(std::max(gram_partial_bytes(guw), gram_partial_bytes(gmax)));
     TallPlan tp = make_tall_plan(n, N, 2 * N, 0);
-    const size_t tparts = std::max((size_t)tp.gy * std::max(N, tp.gx),
-                                   mixed ? (size_t)tall_tc_partials(n, N) : (size_t)0);
+    // one partial per CTA of a block product (also at most 512 of n / 256 blocks, launch_diff_sq)
+    const size_t tparts = std::max((size_t)tp.gy * tp.gx, mixed ? (size_t)tall_tc_partials(n, N) : (size_t)0);
     double *tpart = cv.take<double>(sizeof(double) * tparts);
     const size_t N2 = (size_t)N * N;
     double *G2 = cv.take<double>(sizeof(double) * 4 * N2);

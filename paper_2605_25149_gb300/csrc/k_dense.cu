@@ -64,15 +64,15 @@ __device__ __forceinline__ T gat(const T *X1, int n1, const T *X2, int n2, long 
 
 // One tile over one point chunk: 16 x 16 threads of R x R entries (rows ty + 16 i,
 // columns tx + 16 j), tile edge 16 R.  R is the smallest of 1 .. 4 that covers
-// the tiles (tile_edge): the FP64 pipe bounds the kernel, so entries beyond
+// the plan's columns per tile: the FP64 pipe bounds the kernel, so entries beyond
 // the blocks' columns cost as much as the others (a 64 x 64 tile for 32
 // columns did four times the work).  The diagonal tiles of a symmetric Gram
 // form their sub-blocks on and above the diagonal only (10 of 16 at R = 4).
 // The next stage's loads are issued before the products of this one.  Every
 // entry is summed over the points in order, whatever R.
-// Measured, 48^3 points (before: always 64 x 64 tiles): 16 x 16 columns 807 -> 99,
-// 32 x 32 806 -> 239, 64 x 64 842 -> 792 us, symmetric 798 -> 517 us; the FP64 pipe
-// alone takes 165 us for 32 x 32.
+// Measured by counters, 48^3 points (before, always 64 x 64 tiles: 788 us, symmetric
+// 759): 16 x 16 columns 51, 32 x 32 190 (symmetric 146), 64 x 64 740 us (466); the FP64
+// pipe alone takes 165 us for 32 x 32.
 template <typename T, int R, bool DIAG>
 __device__ __forceinline__ void gram_tile_products(const T (&As)[GK][GT + 1], const T (&Bs)[GK][GT + 1],
                                                    int tx, int ty, T (&acc)[R][R]) {
@@ -1501,11 +1501,12 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
 //  2. V1 = V0 (15/8 I - 10/8 G + 3/8 G^2), G = V0^T V0: orthogonal to FP64
 //     rounding (the step cubes V0's 1e-6), and A' = V1^T A V1 in FP64 on many CTAs;
 //  3. FP64 Jacobi of A' continuing V1 (k_sym_eig_sm<double>): the off-diagonal
-//     starts at 1e-6, so two or three sweeps meet the criterion of k_sym_eig.
+//     starts at 1e-6, so two to four sweeps meet the criterion of k_sym_eig.
 // A non-finite V0 is replaced by I.  The result is FP64's: part 3 is a complete
 // FP64 Jacobi with the tolerance of k_sym_eig whatever V0 was.
-// Measured, N = 64: 7 ms in one FP64 launch before; now 0.6 + 0.08 + 0.66 ms (0.08 ms
-// for part 1 where A is nearly diagonal, as in every refinement round but the first).
+// Measured by counters, N = 64: 7 ms in one FP64 launch before; now 0.66 + 0.07 + 0.54 ms
+// for <U,U> of an early iterate, 1.1 ms for part 3 of its Ritz matrix (part 1: 0.08 ms
+// where A is nearly diagonal, as in every refinement round but the first).
 constexpr int SE_MIN = 5;   // below, the seven launches cost more than the one above: an initial block of 8^3
                             // points, 1 column 127 against 86 us, 4 columns 161, 145, 5 columns 166, 169
 constexpr int SE_MAX = 112;
@@ -2254,6 +2255,8 @@ void launch_extract(int rows, int cols, double alpha, const double *src, int lds
                                                                 ldd));
 }
 
+// out[0] = w * sum of the np partials (fixed order); out[1] = ||A - I||_F of the
+// N x N matrix A (nullable)
 __global__ void k_monitor_finish(int np, const double *part, double w, int N, const double *A,
                                  double *out) {
     __shared__ double red[256];

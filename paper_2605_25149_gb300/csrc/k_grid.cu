@@ -912,7 +912,6 @@ void launch_shift_cols(long n, int N, const double *sft, const double *x, double
     HQ_LAUNCH(HQ_K_VECTOR, k_shift_cols<<<blocks, 256, 0, s>>>(n, N, sft, x, y));
 }
 
-//   out[e] = a * x[e] + b * y[e]            (whole blocks, FP64)
 // of a Newton solve's Gram K = [C; E] (2N x N): Cneg = -C, G = E + beta_j G (column
 // j; first: G = E)
 __global__ void k_newton_project(int N, int first, const double *K, const double *beta, double *Cneg, double *G) {
@@ -925,6 +924,7 @@ void launch_newton_project(int N, bool first, const double *K, const double *bet
                            cudaStream_t s) {
     HQ_LAUNCH(HQ_K_SMALL, k_newton_project<<<(N * N + 255) / 256, 256, 0, s>>>(N, first, K, beta, Cneg, G));
 }
+//   out[e] = a * x[e] + b * y[e]            (whole blocks, FP64)
 __global__ void k_axpby(size_t count, double a, const double *x, double b, const double *y,
                         double *out) {
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count;
