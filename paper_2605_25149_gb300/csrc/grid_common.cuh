@@ -32,7 +32,7 @@ __device__ __forceinline__ float sum6(const float (&x)[6], const bool (&in)[6]) 
 // FP64 pipe for 280 clocks per warp (measured), more than half of every FP64
 // sweep; the same sum takes about 100 integer-ALU instructions (200 clocks) on
 // another pipe than the products around it.  Measured: the operator at 64^3,
-// 64 columns 272 -> 131 us (FP64 pipe 66%, integer ALU 73% busy), an FP64
+// 64 columns 272 -> 130 us (FP64 pipe 68%, integer ALU 75% busy), an FP64
 // block PCG at 64^3, 32 columns 10.9 -> 8.1 ms.  Moving the shifts and
 // additions to the FMA pipe as wide multiply-adds was slower (240 against 198
 // clocks per sum).  The terms are aligned to the largest
