@@ -1015,9 +1015,10 @@ hq_status pcg(hq_ctx *x, const T *B, T *X, double rtol, int maxit, int *iters_ho
             HQ_CUDA(cudaMemcpyAsync(it, x->sc.num_active, sizeof(it), cudaMemcpyDeviceToHost, x->st));
             if (iters_host)
                 HQ_CUDA(cudaMemcpyAsync(iters_host, x->sc.iters, sizeof(int) * x->N, cudaMemcpyDeviceToHost, x->st));
-            HQ_TRY(sync_status(x, x->sc.status, "inner PCG"));
-            x->stat_solves++;
+            const hq_status st = sync_status(x, x->sc.status, "inner PCG");
+            x->stat_solves++;   // failed solves count too
             x->stat_iters += it[1];
+            HQ_TRY(st);
             if (it[0] > 0 && maxit > 0 && rtol > 0.0)
                 return fail(x, HQ_ERR_NOT_CONVERGED, "inner PCG reached cg_maxit");
             return HQ_OK;

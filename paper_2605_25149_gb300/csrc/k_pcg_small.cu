@@ -534,12 +534,12 @@ __global__ void __launch_bounds__(VC_THREADS)
         ps_dot(n, TY, ppt, gy, at_p, w, w, rows, st, [&](double s) {
             if (!(s > 0.0) || !isfinite(s)) {
                 atomicOr(sc.status, ST_BREAKDOWN);
-                go = 0;
+                go = -1;
             } else {
                 step = rz / s;
             }
         });
-        if (!go) break;
+        if (go < 0) break;
         const double alpha = step;
         // x += alpha p, r -= alpha q, |r|
 #pragma unroll
@@ -568,14 +568,17 @@ __global__ void __launch_bounds__(VC_THREADS)
 }
 
 // after k_pcg_small: num_active[0] = columns still active, num_active[1] =
-// iterations of the slowest column; counters (nullable) += those iterations;
+// iterations of the slowest column (with the one a column broke down in: active
+// < 0, cleared here); counters (nullable) += those iterations;
 // ST_PCG_MAXIT for columns that reached the cap (check)
 __global__ void __launch_bounds__(256) k_pcg_small_end(int N, PcgScalars sc, long long *counters, int check) {
     __shared__ int act_sh[8], it_sh[8];
     int act = 0, it = 0;
     for (int c = threadIdx.x; c < N; c += 256) {
-        act += sc.active[c];
-        it = max(it, sc.iters[c]);
+        const int a = sc.active[c];
+        act += a > 0;
+        it = max(it, sc.iters[c] + (a < 0));
+        if (a < 0) sc.active[c] = 0;
     }
     act = __reduce_add_sync(0xffffffffu, act);
     it = __reduce_max_sync(0xffffffffu, it);

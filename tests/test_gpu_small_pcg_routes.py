@@ -86,3 +86,27 @@ def test_batch_member_at_its_iteration_cap(monkeypatch):
     with pytest.raises(hq.HQError) as e:
         hq.Batch([a, b]).step(2)
     assert e.value.status == NOT_CONVERGED and "problem 0" in str(e.value)
+
+
+@pytest.mark.parametrize("scale,rtol,maxit", [(1.0, 1e-9, 1), (1.0, 0.0, 60), (1e-42, 1e-9, 60), (np.nan, 1e-9, 20),
+                                              (np.inf, 0.0, 3), (1e200, 1e-9, 20), (1.0, 1e-9, 0)])
+def test_failed_solves_are_counted(monkeypatch, scale, rtol, maxit):
+    """At the cap, broken down at rounding level (rtol 0; right-hand sides that vanish in FP32),
+    with a non-finite value: status and hq_pcg_stats as of the separate kernels."""
+    m, N = 9, 3
+    B = np.random.default_rng(0).standard_normal((m ** 3, N))
+    if np.isfinite(scale):
+        B *= scale
+    else:
+        B[5, 1] = scale
+    out = []
+    for fused in (True, False):
+        s = context(monkeypatch, m, N, fused)
+        s.profile()
+        try:
+            s.block_pcg(dev(B), rtol=rtol, maxit=maxit)
+            status = 0
+        except hq.HQError as e:
+            status = e.status
+        out.append((status, s.pcg_stats()))
+    assert out[0] == out[1] and out[0][1][0] == 1
