@@ -1369,7 +1369,8 @@ void launch_axpy_small(int count, double a, const double *x, double *y, cudaStre
 // Cyclic Jacobi with a parallel (round-robin) ordering, one CTA.  work: 2 N^2
 // (+ padding to even order).  Rotation: theta = (a_qq - a_pp) / (2 a_pq),
 // t = sign(theta) / (|theta| + sqrt(theta^2 + 1)), c = 1/sqrt(t^2 + 1), s = t c,
-// A <- J^T A J, V <- V J with J = [c s; -s c] on (p, q).
+// A <- J^T A J, V <- V J with J = [c s; -s c] on (p, q).  A is scaled by a power of two
+// first: the squares of the stopping test overflow beyond 1e154.
 __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, double *work,
                                                   double *evals, double *evecs) {
     extern __shared__ double sh[];
@@ -1382,10 +1383,23 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
     int *qq = pp + P / 2;                // P/2
     double *red = (double *)(pp + P);    // 1024 (pp + P is 8-byte aligned: P even)
     const int tid = threadIdx.x, T = blockDim.x;
+    double big = 0.0;
+    for (long idx = tid; idx < (long)N * N; idx += T) big = fmax(big, fabs(Ain[idx]));
+    // over the warp, then over the 32 warps' maxima in every warp
+    for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if ((tid & 31) == 0) red[tid >> 5] = big;
+    __syncthreads();
+    big = red[tid & 31];
+    for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    // 2^-e and 2^e of 2^e <= big < 2^(e+1) (1 for zero, subnormal, infinite or NaN)
+    const int be = (__double2hiint(big) >> 20) & 0x7FF;
+    const bool scaled = be >= 1 && be <= 2045;
+    const double sc = scaled ? __hiloint2double((2046 - be) << 20, 0) : 1.0;
+    const double back = scaled ? __hiloint2double(be << 20, 0) : 1.0;
     for (long idx = tid; idx < (long)P * P; idx += T) {
         int i = (int)(idx / P), j = (int)(idx % P);
         double v = 0.0;
-        if (i < N && j < N) v = 0.5 * (Ain[(size_t)i * N + j] + Ain[(size_t)j * N + i]);
+        if (i < N && j < N) v = 0.5 * (Ain[(size_t)i * N + j] * sc + Ain[(size_t)j * N + i] * sc);
         A[idx] = v;
         Vv[idx] = (i == j) ? 1.0 : 0.0;
     }
@@ -1486,7 +1500,7 @@ __global__ void __launch_bounds__(1024) k_sym_eig(int N, const double *Ain, doub
             double dj = A[(size_t)j * P + j];
             if (dj < di || (dj == di && j < i)) rank++;
         }
-        evals[rank] = di;
+        evals[rank] = di * back;
         if (evecs)
             for (int k = 0; k < N; k++) evecs[(size_t)k * N + rank] = Vv[(size_t)k * P + i];
     }

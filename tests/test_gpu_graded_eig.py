@@ -56,3 +56,22 @@ def test_smallest_eigenvalue_of_a_graded_gram(N, k):
     got, ref = s.monitor()["smin"], smallest_sv2(U * np.sqrt(h3))
     e = 2.0 ** -53 * ((n + 2) * np.abs(Q.T @ Q).max() + 20 * N)
     assert abs(got - ref) <= ref * N * e / np.linalg.eigvalsh(Q.T @ Q)[0]
+
+
+@pytest.mark.parametrize("N", [1, 2, 4, 5, 64, 112, 113])
+@pytest.mark.parametrize("k", [-330, 330])
+def test_scale_of_the_block_is_immaterial(N, k):
+    """Powers of two pass through Gram, eigenvalues and the initial scaling exactly, also where
+    the squares of the Gram's entries leave the exponent range (2^660 and 2^-660)."""
+    m = 6
+    U = np.random.default_rng(N).standard_normal((m ** 3, N))
+    out = []
+    for f in (1.0, 2.0 ** k):
+        s = hq.Solver(m, N)
+        s.set_potential(inputs.harmonic(m))
+        s.set_state(U * f, 0)
+        mon = s.monitor()
+        s.set_initial(U * f)
+        out.append((mon["smin"] / f / f, mon["smax"] / f / f, s.get_state()[0]))
+    assert out[0][:2] == out[1][:2]
+    assert np.array_equal(out[0][2], out[1][2])
